@@ -8,9 +8,10 @@ Sizes are those of the repository's workloads: the tiny grid (32 tau x 64 bins x
 the paper-scale grid (200 x 1000 x 4096), the band example (160 x 1000 x 1500 walkers), the
 precision workload (512 x 2048 x 16384) and the uneven batch (50-500 tau, 200-2000 bins).
 
-The blocks run at temperatures at or above 1e8 in units of chi2, where two anneals whose
-delta chi2 differ in the last bits of FP32 still take every decision alike (no walker of 4096
-parted in 1e9 moves), so that a block's result is a number and not a matter of chance.
+The blocks run at temperatures of the order of the residue, as the first half of a schedule
+does: there a decision lies further from its threshold than FP32's rounding (and its drift over
+the sweeps between two recomputations) reaches, so that a block's result is a number and not a
+matter of which last bit a chain of 1e8 decisions met.
 """
 import math
 
@@ -39,7 +40,7 @@ def listed():
         {"name": "block_paper", **block, "n_tau": 200, "n_omega": 1000, "walkers": 4096},
         # a block of the schedule that reaches the noise level (absolute temperatures, finer
         # moves), part way down: fewer proposals fail the positivity test
-        {"name": "block_cooled", **block, "n_tau": 200, "n_omega": 1000, "walkers": 4096, "T_start_abs": 1e9,
+        {"name": "block_cooled", **block, "n_tau": 200, "n_omega": 1000, "walkers": 4096, "T_start_abs": 1e12,
          "T_end_abs": 0.03, "scale": 0.1},
         # the band example: few walkers, self-cooling, adaptive branching, smoothing
         {"name": "block_band", **block, "n_tau": 160, "n_omega": 1000, "walkers": 1500, "tau_max": 7.95, "w_max": 3.5,
