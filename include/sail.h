@@ -147,7 +147,11 @@ typedef struct sail_params {
                                look-ahead's in the last bits); 0 = choose: look-ahead when the problem has
                                at least 16 walkers per SM (measured faster there, slower with fewer)
                                and the last block rejected at least 30% of its proposals for
-                               positivity (measured +12% at 40%, -6% at 22-27%) */
+                               positivity (measured +12% at 40%, -6% at 22-27%).  Own-bin blocks in
+                               which no decision is expected within FP32's rounding of its
+                               threshold run a third loop whatever lanes and loop are chosen: the
+                               same draws and decisions, delta chi2 summed in an orthonormal basis
+                               of the kernel's columns (16 to 32 terms instead of n_tau) */
     double T_start_abs;     /* > 0: the geometric schedule starts at this absolute temperature
                                instead of T_start chi2_0 (skip the boiling far above the data's
                                scale, whatever chi2_0 is); 0 = T_start */

@@ -22,6 +22,12 @@ UNITS = {
     "api.cu": [],
     "exact64.cu": ["-fmad=false"],
     "sweep_fp32.cu": [],
+    "span.cu": ["-fmad=false"],
+    "sweep_span16.cu": [],
+    "sweep_span24.cu": [],
+    "sweep_span32.cu": [],
+    "sweep_span_batch.cu": [],
+    "sweep_span_batch_modes.cu": [],
     "sweep_walk.cu": [],
     "sweep_hastings.cu": [],
     "sweep_guard.cu": [],

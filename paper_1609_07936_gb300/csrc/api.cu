@@ -77,6 +77,7 @@ struct Layout {
     size_t pr_walker, pr_p, pr_s, pr_eps, pr_delta, pr_ok;
     size_t tma_a, tma_b;     // pre-tiled BF16 pieces of the spectra and the kernel table (resync kind 2)
     size_t chi2_all;         // chi2 of the whole population (sail_branch_solve)
+    size_t Kspan, Uspan, Fspan, U64, span_worst;   // the kernel columns' basis (FP32, sweep_span.cuh)
     size_t total;
     int max_events;
 };
@@ -155,6 +156,13 @@ Layout make_layout(int n_tau, int n_omega, const sail_params &p) {
     L.pr_ok = take((size_t)kProbeMax * 4);
     L.x4_32 = take(NO * 16);
     L.mrho32 = take(PAD * 4);
+    if (p.precision == SAIL_PREC_FP32) {
+        L.Kspan = take(NO * kSpanMax * 4);
+        L.Uspan = take(PAD * kSpanMax * 8);
+        L.Fspan = take(kSpanMax * 4);
+        L.U64 = take(PAD * kSpanMax * 8);
+        L.span_worst = take(8);
+    }
     L.total = off;
     return L;
 }
@@ -247,6 +255,8 @@ struct sail_ctx {
     int *status;             // device status word: nonzero after a timed-out device wait
     bool ahead_auto;         // FP32 sweep_loop 0 with enough walkers: the loop follows the rejections
     double pos_frac_last = -1.0;   // positivity-rejected share of the last block's proposals
+    double chi2_ref;         // mean chi2 of the walkers before the next block (NaN: not known)
+    double F_norm;           // |F / sigma|
     bool converged;          // chi2 of the averaged spectrum reached target_chi2
     double chi2_of_mean;
     // optional per-kernel timing: event pairs recorded around launches, read at block ends
@@ -272,6 +282,26 @@ constexpr double kAheadMinPos = 0.30;
 int sweep_ahead_next(const sail_ctx *h) {
     if (h->ahead_auto && h->pos_frac_last >= 0.0) return h->pos_frac_last >= kAheadMinPos ? 1 : 0;
     return h->P.ahead;
+}
+
+// Whether the next block's sweeps [n0, n1) run in the span of the kernel's columns
+// (sweep_span.cuh) or over tau.  The two round delta chi2 differently, and a decision that lies
+// within that rounding of its threshold can come out differently; at a low temperature one such
+// decision parts a walker from its chain, and branching the population from its result.  So that a
+// run gives the same result either way, the span sweep takes the blocks in which such a decision
+// is not expected: moves x 1e-7 x S / T of them, 1e-7 the rounding of delta chi2 (and its drift
+// between two recomputations) relative to the magnitude of its terms, S = eps_max |R| (|R| + |Fhat|)
+// that magnitude.  Measured on the paper-scale problem, walkers of 4096 that parted in a block of
+// 4.1e8 moves: 0 at T = 10 chi2_0 .. 0.5 chi2_0 (estimate 0.004 .. 0.06), 7 to 17 at T = 1e6 near
+// equilibrium (estimate 16); the line is drawn at 1/16 of a decision a block.
+bool span_next(const sail_ctx *h, int n0, int n1) {
+    const sail_params &p = h->prm;
+    if (h->P.span == 0 || p.shared_bins > 1 || p.fp64_accept) return false;
+    const double T = std::min(h->T[n0], h->T[n1 - 1]);
+    const double eps = p.move_scale > 0.0 ? p.move_scale : 1.0 / h->n_omega;
+    const double R = std::sqrt(h->chi2_ref), S = eps * R * (R + h->F_norm);
+    const double moves = (double)(n1 - n0) * p.n_walkers * h->n_omega;
+    return moves * 1e-7 * std::min(1.0, S / T) <= 0.0625;     // chi2 not known (NaN): S / T counts as 1
 }
 
 // A named NVTX range around the host calls that enqueue one phase of the schedule (sweep,
@@ -312,6 +342,49 @@ void timed_collect(sail_ctx *h) {
         }
     }
     h->n_timed = 0;
+}
+
+// The basis of the kernel's columns for the FP32 sweep: from 64 sampled columns, and where those miss
+// some column (checked on the device), from up to 256.  Where 32 directions do not hold every column
+// the handle keeps span = 0 and the sweeps over tau.
+cudaError_t span_init(sail_ctx *h, const std::vector<double> &K64, const std::vector<double> &F64) {
+    DevProblem &P = h->P;
+    const int PAD = h->pad;
+    char *ws = h->ws;
+    std::vector<double> U;
+    for (int samples : {64, 256}) {
+        const int rr = span_basis(K64.data(), h->n_tau, PAD, h->n_omega, samples, U);
+        if (rr == 0) continue;
+        std::vector<float> U32((size_t)h->n_tau * rr * 2), Fs(rr);
+        for (int k = 0; k < rr; ++k) {
+            double f = 0.0;
+            for (int i = 0; i < h->n_tau; ++i) {
+                const double u = U[(size_t)k * PAD + i];
+                f += u * F64[i];
+                U32[2 * ((size_t)i * rr + k)] = (float)u;
+                U32[2 * ((size_t)i * rr + k) + 1] = (float)(u - (double)(float)u);
+            }
+            Fs[k] = (float)f;
+        }
+        P.span = rr;
+        P.Kspan = (const float *)(ws + h->L.Kspan);
+        P.Uspan = (const float *)(ws + h->L.Uspan);
+        P.Fspan = (const float *)(ws + h->L.Fspan);
+        cudaError_t e = cudaMemcpyAsync(ws + h->L.U64, U.data(), U.size() * 8, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ws + h->L.Uspan, U32.data(), U32.size() * 4, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ws + h->L.Fspan, Fs.data(), Fs.size() * 4, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess)
+            e = launch_span_table(P, (const double *)(ws + h->L.U64), (float *)(ws + h->L.Kspan),
+                                  (double *)(ws + h->L.span_worst), h->stream);
+        double worst = 0.0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&worst, ws + h->L.span_worst, 8, cudaMemcpyDeviceToHost, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        h->launches += 1;
+        if (e != cudaSuccess) return e;
+        if (span_fits(worst)) return cudaSuccess;
+        P.span = 0;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -542,6 +615,10 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     h->B = B;
     h->lambda0 = lambda;
     h->chi2_0 = chi2_0;
+    h->chi2_ref = chi2_0;
+    h->F_norm = 0.0;
+    for (int i = 0; i < n_tau; ++i) h->F_norm += F64[i] * F64[i];
+    h->F_norm = std::sqrt(h->F_norm);
     h->stream = (cudaStream_t)stream;
     h->ws = (char *)d_workspace;
     h->ws_bytes = ws_bytes;
@@ -660,6 +737,7 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     if (e == cudaSuccess)
         e = launch_init_state(P, S, p->precision, (const double *)(ws + L.a0), (const double *)(ws + L.R0), chi2_0, st);
     h->launches = 1;
+    if (e == cudaSuccess && p->precision == SAIL_PREC_FP32) e = span_init(h, K64, F64);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         delete h;
@@ -918,6 +996,7 @@ int block_finish(sail_ctx *h, const BlockPending &b, sail_block_stats *out) {
         const double proposed = (double)(b.block_end - b.n_begin) * p.n_walkers * h->n_omega;
         h->pos_frac_last = (double)(b.bc.pos - h->pos_seen) / proposed;
     }
+    h->chi2_ref = b.bc.chi2_sum / p.n_walkers;
     h->acc_seen = b.bc.acc;
     h->pos_seen = b.bc.pos;
     h->blocks_done += 1;
@@ -950,6 +1029,7 @@ int sail_anneal(sail_t h, int max_blocks, sail_block_stats *stats, int *n_done) 
         BlockPending b{};
         b.n_begin = h->sweeps_done;
         b.block_end = block_end_of(h);
+        h->P.span_on = p.precision == SAIL_PREC_FP32 && span_next(h, b.n_begin, b.block_end);
         for (int n = b.n_begin; n < b.block_end;) {
             const int next = next_resync(h, n, b.block_end);
             const int tk = timed_begin(h);
@@ -1034,6 +1114,7 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev) {
     SAIL_CUDA(launch_resync(h->P, h->S, h->prm.precision, 0, h->prm.resync_kind, h->status, st, &l), "resync launch");
     h->launches += l;
     SAIL_CUDA(cudaStreamSynchronize(st), "set_state sync");
+    h->chi2_ref = NAN;
     return SAIL_OK;
 }
 
@@ -1258,6 +1339,14 @@ int sail_restore(sail_t h, const void *buf, size_t bytes) {
     in += (size_t)h->prm.n_sweeps * 8;
     for (const CkptRegion &r : ckpt_regions(h)) {
         SAIL_CUDA(cudaMemcpyAsync(h->ws + r.off, in, r.bytes, cudaMemcpyHostToDevice, h->stream), "restore H2D");
+        if (r.off == h->L.chi2) {
+            double sum = 0.0, c2;
+            for (int w = 0; w < h->prm.n_walkers; ++w) {
+                std::memcpy(&c2, in + (size_t)w * 8, 8);
+                sum += c2;
+            }
+            h->chi2_ref = sum / h->prm.n_walkers;
+        }
         in += r.bytes;
     }
     SAIL_CUDA(cudaStreamSynchronize(h->stream), "restore sync");
@@ -1341,9 +1430,11 @@ struct sail_batch_ctx {
     BatchItem *d_items;
     int *d_counter;
     size_t max_items;
-    // a batched sweep segment launches one kernel per class of problems: lanes per walker
-    // (16 or 8) times move-loop variant (plain, walk, Hastings); class = 3 * (lanes == 8) + mode
-    static constexpr int kClasses = 6;
+    // a batched sweep segment launches one kernel per class of problems: the sweeps over tau by
+    // lanes per walker (16 or 8), or the span sweep, times move-loop variant (plain, walk,
+    // Hastings); class = 3 * (lanes == 8) + mode, or 6 + mode for the span sweep
+    static constexpr int kClasses = 9;
+    int span_lanes;            // lanes per walker of the plain span class in this segment (4 or 8)
     size_t smem[kClasses];     // shared memory of each class's kernel: its problems' largest tables
     cudaStream_t aux[kClasses - 1];   // further streams: the classes' kernels run side by side
     cudaEvent_t fork, join[kClasses - 1];
@@ -1382,7 +1473,22 @@ int check_batch(int n, const sail_problem *probs) {
     return SAIL_OK;
 }
 
-int batch_class(const DevProblem &P) { return 3 * (P.lanes == 8 ? 1 : 0) + sweep_mode(P); }
+int batch_class(const DevProblem &P) {
+    if (P.span_on) return 6 + sweep_mode(P);
+    return 3 * (P.lanes == 8 ? 1 : 0) + sweep_mode(P);
+}
+
+// Shared memory that a problem may ask of its classes' kernels (it changes between the sweep over
+// tau and the span sweep from block to block).
+void batch_reserve(size_t *smem, const DevProblem &P) {
+    int dev = 0, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const int mode = sweep_mode(P);
+    size_t &tau = smem[3 * (P.lanes == 8 ? 1 : 0) + mode], &span = smem[6 + mode];
+    tau = std::max(tau, sweep_fp32_table_bytes(P));
+    if (P.span > 0) span = std::max(span, span_batch_smem(P, smem_max));
+}
 
 void batch_streams_create(sail_batch_ctx *b) {
     cudaEventCreate(&b->ev0);
@@ -1422,8 +1528,12 @@ cudaError_t batch_sweep_segment(sail_batch_ctx *b, const int *count) {
     for (int c = 0; c < sail_batch_ctx::kClasses; ++c) {
         if (count[c] == 0) continue;
         cudaStream_t sc = k == 0 ? st : b->aux[k - 1];
-        e = launch_sweep_batch(b->d_probs, b->d_items + offset, count[c], b->d_counter + c, b->smem[c], b->item_pairs,
-                               c >= 3 ? 8 : 16, c % 3, sc);
+        if (c >= 6)
+            e = launch_span_batch(b->d_probs, b->d_items + offset, count[c], b->d_counter + c, b->smem[c], b->item_pairs,
+                                  b->span_lanes, c - 6, sc);
+        else
+            e = launch_sweep_batch(b->d_probs, b->d_items + offset, count[c], b->d_counter + c, b->smem[c], b->item_pairs,
+                                   c >= 3 ? 8 : 16, c % 3, sc);
         if (e != cudaSuccess) return e;
         offset += count[c];
         ++k;
@@ -1489,8 +1599,7 @@ int sail_batch_create(sail_batch_t *out, int n, const sail_problem *probs, int a
             return rc;
         }
         b->h.push_back(h);
-        size_t &sm = b->smem[batch_class(h->P)];
-        sm = std::max(sm, sweep_fp32_table_bytes(h->P));
+        batch_reserve(b->smem, h->P);
         off += align_up(sub);
     }
     b->autotune = autotune;
@@ -1562,13 +1671,18 @@ int batch_run_blocks(sail_batch_ctx *b, int max_blocks, int *n_done) {
             pend[k] = BlockPending{};
             pend[k].n_begin = b->h[k]->sweeps_done;
             pend[k].block_end = block_end_of(b->h[k]);
+            b->h[k]->P.span_on = span_next(b->h[k], pend[k].n_begin, pend[k].block_end);
             cur[k] = pend[k].n_begin;
         }
         if (!any) break;
         for (;;) {
             // one segment: every problem with sweeps left in this block advances to its next resync
             for (auto &v : cls_items) v.clear();
-            long long seg_moves = 0;
+            long long seg_moves = 0, span_walkers = 0;
+            for (int k = 0; k < N; ++k)
+                if (active[k] && cur[k] < pend[k].block_end && batch_class(b->h[k]->P) == 6)
+                    span_walkers += b->h[k]->prm.n_walkers;
+            b->span_lanes = span_batch_lanes(span_walkers);
             for (int k = 0; k < N; ++k) {
                 sail_ctx *h = b->h[k];
                 hp[k].n0 = hp[k].n1 = 0;
@@ -1578,12 +1692,13 @@ int batch_run_blocks(sail_batch_ctx *b, int max_blocks, int *n_done) {
                 hp[k].n0 = cur[k];
                 hp[k].n1 = next_resync(h, cur[k], pend[k].block_end);
                 seg_moves += (long long)(hp[k].n1 - hp[k].n0) * h->prm.n_walkers * h->n_omega;
-                const int wpw = sweep_walkers_per_warp(h->P);
+                const int cls = batch_class(h->P);
+                const int wpw = cls >= 6 ? 32 / (cls == 6 ? b->span_lanes : 8) : sweep_walkers_per_warp(h->P);
                 const int groups = (h->prm.n_walkers + wpw - 1) / wpw;
-                // walker groups per item = warps per block (at most 8 with 8 lanes per walker, 12
-                // with 16)
-                const int per = std::min(b->item_pairs, h->P.lanes == 8 ? 8 : 12);
-                std::vector<BatchItem> &dst = cls_items[batch_class(h->P)];
+                // walker groups per item = warps per block (over tau at most 8 with 8 lanes per walker,
+                // 12 with 16; span sweep 16)
+                const int per = cls >= 6 ? b->item_pairs : std::min(b->item_pairs, h->P.lanes == 8 ? 8 : 12);
+                std::vector<BatchItem> &dst = cls_items[cls];
                 for (int lo = 0; lo < groups; lo += per) dst.push_back(BatchItem{k, lo, std::min(lo + per, groups)});
             }
             int count[sail_batch_ctx::kClasses];
@@ -1825,8 +1940,7 @@ int server_step(sail_server_t s, int *completed, int max_completed, int *n_compl
             return rc;
         }
         b.h[slot] = h;
-        size_t &sm = b.smem[batch_class(h->P)];
-        sm = std::max(sm, sweep_fp32_table_bytes(h->P));
+        batch_reserve(b.smem, h->P);
         s->slot_off[slot] = off;
         s->slot_size[slot] = r.bytes;
         s->slot_id[slot] = r.id;

@@ -16,6 +16,7 @@
 //   R64 / R32        [n_walkers][n_tau_pad] residuals, zero past n_tau
 #pragma once
 #include <cstdint>
+#include <vector>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -71,6 +72,11 @@ struct DevProblem {
     int fp64_accept;       // FP32: 1 = decisions near the threshold taken again in FP64, 2 = all of them
     const float *x4_32;    // uniform tau grid: per-bin powers of X_j (8-lane sweep's columns)
     const float *mrho32;   // uniform tau grid: minus the ratio of Khat_{i,0} to its quad's first
+    int span;              // FP32: directions of the kernel columns' basis (16, 24 or 32), 0: none (sweep_span.cuh)
+    int span_on;           // this block's sweeps run in that basis
+    const float *Kspan;    // [n_omega][span] the columns in that basis
+    const float *Uspan;    // [n_tau][span][2] the basis, each entry a pair of floats
+    const float *Fspan;    // [span] Fhat in that basis
 };
 
 struct DevState {
@@ -115,6 +121,17 @@ cudaError_t launch_sweep_fp64(const DevProblem &P, const DevState &S, int sweep_
                               int sweep_end, cudaStream_t st);
 cudaError_t launch_sweep_fp32(const DevProblem &P, const DevState &S, int sweep_begin,
                               int sweep_end, cudaStream_t st);
+// The FP32 sweep in the span of the kernel's columns (P.span_on); launch_sweep_fp32 calls it.
+constexpr int kSpanMax = 32;
+inline int span_width(int need) { return need <= 16 ? 16 : need <= 24 ? 24 : 32; }
+cudaError_t launch_sweep_span(const DevProblem &P, const DevState &S, int sweep_begin, int sweep_end, cudaStream_t st);
+// An orthonormal basis of the columns Khat (K64: [n_omega][pad]) from n_samples of them, U[kSpanMax][pad]
+// (unused directions zero); returns its width (16, 24 or 32), or 0 where 32 directions do not do.
+int span_basis(const double *K64, int n_tau, int pad, int n_omega, int n_samples, std::vector<double> &U);
+// Kspan from P.Khat64 and the basis, and the largest part of a column that the basis leaves, relative
+// to its norm (device); span_fits says whether that is small enough.
+cudaError_t launch_span_table(const DevProblem &P, const double *U, float *Kspan, double *worst, cudaStream_t st);
+bool span_fits(double worst);
 // The FP32 sweep of a problem with an index walk (P.walk_len > 0); launch_sweep_fp32 calls it.
 cudaError_t launch_sweep_walk(const DevProblem &P, const DevState &S, int sweep_begin, int sweep_end,
                               cudaStream_t st);
@@ -198,6 +215,13 @@ cudaError_t launch_sweep_batch(const BatchProblem *d_probs, const BatchItem *d_i
                                size_t smem, int warps, int lanes, int mode, cudaStream_t st);
 cudaError_t launch_sweep_batch8(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                 size_t smem, int warps, int mode, cudaStream_t st);
+// The batched span sweep of problems whose P.span_on is set (any widths together): blocks of `warps`
+// warps (at most 16), lanes (4 or 8) per walker for the plain mode (8 for the others; the results do
+// not depend on it), smem at least the problems' span_batch_smem.
+size_t span_batch_smem(const DevProblem &P, int smem_max);
+int span_batch_lanes(long long walkers);
+cudaError_t launch_span_batch(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
+                              size_t smem, int warps, int lanes, int mode, cudaStream_t st);
 cudaError_t launch_read_probe(const void *buf, size_t bytes, int reps, void *sink, cudaStream_t st);
 cudaError_t launch_smem_probe(int reps, void *sink, cudaStream_t st, double *bytes);
 
