@@ -73,7 +73,7 @@ struct Layout {
     size_t a64, b32, g2, R64, R32, chi2, acc_prev, hash, n_acc, n_pos, guard;
     size_t acc_trace, m_trace, delta_trace;
     size_t m, zero_l, donor_l, n_pairs, delta, counters, bz, bxi, cand, cand_Z, ctl;
-    size_t mean, err, R_mean, chi2_mean, n_used, cut;
+    size_t mean, err, R_mean, chi2_mean, n_used, cut, avg_idx, avg_parts;
     size_t pr_walker, pr_p, pr_s, pr_eps, pr_delta, pr_ok;
     size_t tma_a, tma_b;     // pre-tiled BF16 pieces of the spectra and the kernel table (resync kind 2)
     size_t chi2_all;         // chi2 of the whole population (sail_branch_solve)
@@ -148,6 +148,8 @@ Layout make_layout(int n_tau, int n_omega, const sail_params &p) {
     L.chi2_mean = take(8);
     L.n_used = take(4);
     L.cut = take(8);
+    L.avg_idx = take(W * 4);
+    if (p.precision == SAIL_PREC_FP32) L.avg_parts = take((size_t)2 * kAvgChunks * NO * 8);
     L.pr_walker = take((size_t)kProbeMax * 4);
     L.pr_p = take((size_t)kProbeMax * 4);
     L.pr_s = take((size_t)kProbeMax * 4);
@@ -802,7 +804,8 @@ int average_to_host(sail_t h, double *mean, double *err, int *n_used, double *ch
     int l = 0;
     cudaError_t e = launch_average(h->P, h->S, h->prm.precision, h->prm.avg_chi2_factor,
                                    (double *)(ws + h->L.mean), (double *)(ws + h->L.err), (int *)(ws + h->L.n_used),
-                                   (double *)(ws + h->L.cut), (double *)(ws + h->L.R_mean),
+                                   (double *)(ws + h->L.cut), (int *)(ws + h->L.avg_idx),
+                                   (double *)(ws + h->L.avg_parts), (double *)(ws + h->L.R_mean),
                                    (double *)(ws + h->L.chi2_mean), h->stream, &l);
     h->launches += l;
     if (e != cudaSuccess) return cuda_fail(e, "average");

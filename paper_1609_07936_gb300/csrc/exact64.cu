@@ -811,63 +811,171 @@ __global__ void block_stats_kernel(DevProblem P, DevState S, BlockCounters *out)
 }
 
 // ------------------------------------------------------------------ stochastic average
-// Walkers with chi2 <= factor * min chi2; mean over them (walkers ascending) and the standard
-// error sqrt(sum (a - mean)^2 / (n - 1)) / sqrt(n) per bin (Sec. 1).
-__global__ void average_select_kernel(DevProblem P, DevState S, double factor, int *n_used,
-                                      double *cut_out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double cmin = S.chi2[0];
-    for (int w = 1; w < P.n_walkers; ++w) if (S.chi2[w] < cmin) cmin = S.chi2[w];
+// Walkers with chi2 <= factor * min chi2; mean over them and the standard error
+// sqrt(sum (a - mean)^2 / (n - 1)) / sqrt(n) per bin (Sec. 1).
+//
+// One block selects: the smallest chi2 (a NaN in walker 0's place stands, elsewhere it is passed
+// over), the cut, and the list of the walkers below it, ascending.  (One thread over all walkers
+// took 0.46 ms at 4096 and 1.8 ms at 16384; the block takes about 10 us.)
+constexpr int kSelectThreads = 1024;
+__global__ void __launch_bounds__(kSelectThreads) average_select_kernel(DevProblem P, DevState S, double factor, int *n_used,
+                                                                        double *cut_out, int *idx) {
+    __shared__ SolveShared sh;
+    const int W = P.n_walkers, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double c0 = S.chi2[0];
+    double cmin = c0;
+    for (int w = tid; w < W; w += kSelectThreads) {
+        const double c = S.chi2[w];
+        cmin = c < cmin ? c : cmin;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double c = __shfl_xor_sync(kFull, cmin, o);
+        cmin = c < cmin ? c : cmin;
+    }
+    if (lane == 0) sh.red_d[warp] = cmin;
+    __syncthreads();
+    cmin = c0;
+    for (int k = 0; k < kSelectThreads / 32; ++k) cmin = sh.red_d[k] < cmin ? sh.red_d[k] : cmin;
     const double cut = factor * cmin;
     int used = 0;
-    for (int w = 0; w < P.n_walkers; ++w) used += (S.chi2[w] <= cut);
-    *n_used = used;
-    *cut_out = cut;
+    for (int w0 = 0; w0 < W; w0 += kSelectThreads) {
+        const int w = w0 + tid;
+        const int in = w < W && S.chi2[w] <= cut;
+        int total;
+        const int at = block_scan_excl(in, &total, sh);
+        if (in) idx[used + at] = w;
+        used += total;
+    }
+    if (tid == 0) {
+        *n_used = used;
+        *cut_out = cut;
+    }
 }
 
-__global__ void average_bins_kernel(DevProblem P, DevState S, int precision, const int *n_used,
-                                    const double *cut_in, double *mean, double *err) {
+// FP64 state: one thread per bin, sums over the selected walkers in ascending order (the
+// validation path's order), eight loads in flight before their eight ordered additions.
+__global__ void __launch_bounds__(32) average_bins64_kernel(DevProblem P, DevState S, const int *n_used, const int *idx,
+                                                            double *mean, double *err) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= P.n_omega) return;
-    const double cut = *cut_in;
     const int used = *n_used;
-    auto at = [&](int w) -> double {
-        if (precision == 0) return S.a64[(size_t)w * P.n_omega + j];
-        return (double)S.b32[(size_t)w * P.n_omega + j];
-    };
-    double m = 0.0;
-    for (int w = 0; w < P.n_walkers; ++w) if (S.chi2[w] <= cut) m += at(w);
-    m /= used;
-    double e = 0.0;
-    if (used > 1) {
-        for (int w = 0; w < P.n_walkers; ++w) {
-            if (!(S.chi2[w] <= cut)) continue;
-            const double v = at(w) - m;
-            e += v * v;
+    const double *a = S.a64 + j;
+    const size_t NO = P.n_omega;
+    auto walk = [&](auto &&term) {
+        int k = 0;
+        for (; k + 8 <= used; k += 8) {
+            double v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = a[(size_t)idx[k + q] * NO];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) term(v[q]);
         }
+        for (; k < used; ++k) term(a[(size_t)idx[k] * NO]);
+    };
+    double m = 0.0, e = 0.0;
+    walk([&](double v) { m += v; });
+    m /= used;
+    if (used > 1) {
+        walk([&](double v) {
+            const double d = v - m;
+            e += d * d;
+        });
         e = sqrt(e / (used - 1)) / sqrt((double)used);
     }
     mean[j] = m;
-    if (err) err[j] = e;
+    err[j] = e;
 }
 
-__global__ void __launch_bounds__(128) residual_of_kernel(DevProblem P, const double *a, double *R,
-                                                          double *chi2) {
-    __shared__ double Rs[kMaxTau];
-    for (int i = threadIdx.x; i < P.n_tau_pad; i += blockDim.x) {
-        double r = 0.0;
-        if (i < P.n_tau) {
-            double model = 0.0;
-            for (int j = 0; j < P.n_omega; ++j) model = model + P.Khat64[(size_t)j * P.n_tau_pad + i] * a[j];
-            r = P.Fhat64[i] - model;
-        }
-        Rs[i] = r;
-        if (R) R[i] = r;
+// FP32 state: FP64 sums over kAvgChunks equal parts of the selected walkers, one block per part
+// and 128 bins, then over the parts in order.  The bound is the FP64 pipe (two conversions, two
+// additions and a fused multiply-add per element at 2 lanes a clock and SM) once enough blocks
+// are in flight; one thread per bin over all walkers was bound by one load's latency at a time
+// (1.48 ms at 4096 x 1000, 4.7 ms at 16384 x 2048).  A whole sail_average call: 2.41 -> 0.24 ms at
+// 200 tau x 1000 bins x 4096 walkers, 9.65 -> 0.37 ms at 512 x 2048 x 16384.
+constexpr int kAvgBins = 128;
+template <bool VAR>
+__global__ void __launch_bounds__(kAvgBins) average_part_kernel(DevProblem P, DevState S, const int *n_used, const int *idx,
+                                                                const double *sums, double *out, double *mean) {
+    const int j = blockIdx.x * kAvgBins + threadIdx.x, part = blockIdx.y;
+    if (j >= P.n_omega) return;
+    const size_t NO = P.n_omega;
+    const int used = *n_used, per = (used + kAvgChunks - 1) / kAvgChunks;
+    const int k0 = min(part * per, used), k1 = min(k0 + per, used);
+    double m = 0.0;
+    if constexpr (VAR) {
+        for (int c = 0; c < kAvgChunks; ++c) m += sums[c * NO + j];
+        m /= used;
+        if (part == 0) mean[j] = m;
     }
+    const float *b = S.b32 + j;
+    double s0 = 0.0, s1 = 0.0;
+    auto term = [&](double &s, float v) {
+        if constexpr (VAR) {
+            const double d = (double)v - m;
+            s = fma(d, d, s);
+        } else {
+            s += (double)v;
+        }
+    };
+    int k = k0;
+    for (; k + 8 <= k1; k += 8) {
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = b[(size_t)idx[k + q] * NO];
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) {
+            term(s0, v[q]);
+            term(s1, v[q + 1]);
+        }
+    }
+    for (; k < k1; ++k) term(s0, b[(size_t)idx[k] * NO]);
+    out[part * NO + j] = s0 + s1;
+}
+
+__global__ void __launch_bounds__(kAvgBins) average_err_kernel(DevProblem P, const int *n_used, const double *squares, double *err) {
+    const int j = blockIdx.x * kAvgBins + threadIdx.x;
+    if (j >= P.n_omega) return;
+    const int used = *n_used;
+    double e = 0.0;
+    if (used > 1) {
+        for (int c = 0; c < kAvgChunks; ++c) e += squares[(size_t)c * P.n_omega + j];
+        e = sqrt(e / (used - 1)) / sqrt((double)used);
+    }
+    err[j] = e;
+}
+
+// Residual of one spectrum: thread i sums the model over the bins in order (eight products in
+// flight ahead of their ordered additions), one warp a block so that every SM's FP64 pipe serves
+// one of them; then one thread sums chi2 in order.  (One block of 128 threads, a load at a time:
+// 0.47 ms at 200 x 1000, 2.0 ms at 512 x 2048.)
+__global__ void __launch_bounds__(32) residual_of_kernel(DevProblem P, const double *a, double *R) {
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    const size_t PAD = P.n_tau_pad;
+    double r = 0.0;
+    if (i < P.n_tau) {
+        const double *K = P.Khat64 + i;
+        double model = 0.0;
+        int j = 0;
+        for (; j + 8 <= P.n_omega; j += 8) {
+            double p[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) p[q] = K[(j + q) * PAD] * a[j + q];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) model = model + p[q];
+        }
+        for (; j < P.n_omega; ++j) model = model + K[j * PAD] * a[j];
+        r = P.Fhat64[i] - model;
+    }
+    R[i] = r;
+}
+__global__ void __launch_bounds__(128) chi2_of_kernel(DevProblem P, const double *R, double *chi2) {
+    __shared__ double Rs[kMaxTau];
+    for (int i = threadIdx.x; i < P.n_tau; i += blockDim.x) Rs[i] = R[i] * R[i];
     __syncthreads();
     if (threadIdx.x == 0) {
         double c2 = 0.0;
-        for (int i = 0; i < P.n_tau; ++i) c2 = c2 + Rs[i] * Rs[i];
+#pragma unroll 8
+        for (int i = 0; i < P.n_tau; ++i) c2 = c2 + Rs[i];
         *chi2 = c2;
     }
 }
@@ -1072,16 +1180,22 @@ cudaError_t launch_block_stats(const DevProblem &P, const DevState &S, BlockCoun
 }
 
 cudaError_t launch_average(const DevProblem &P, const DevState &S, int precision, double factor, double *mean,
-                           double *err, int *n_used, double *cut, double *R_mean, double *chi2_mean,
-                           cudaStream_t st, int *launches) {
-    average_select_kernel<<<1, 32, 0, st>>>(P, S, factor, n_used, cut);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    average_bins_kernel<<<(P.n_omega + 127) / 128, 128, 0, st>>>(P, S, precision, n_used, cut, mean, err);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    residual_of_kernel<<<1, 128, 0, st>>>(P, mean, R_mean, chi2_mean);
-    *launches += 3;
+                           double *err, int *n_used, double *cut, int *idx, double *parts, double *R_mean,
+                           double *chi2_mean, cudaStream_t st, int *launches) {
+    average_select_kernel<<<1, kSelectThreads, 0, st>>>(P, S, factor, n_used, cut, idx);
+    if (precision == 0) {
+        average_bins64_kernel<<<(P.n_omega + 31) / 32, 32, 0, st>>>(P, S, n_used, idx, mean, err);
+        *launches += 4;
+    } else {
+        double *squares = parts + (size_t)kAvgChunks * P.n_omega;
+        const dim3 grid((P.n_omega + kAvgBins - 1) / kAvgBins, kAvgChunks);
+        average_part_kernel<false><<<grid, kAvgBins, 0, st>>>(P, S, n_used, idx, nullptr, parts, nullptr);
+        average_part_kernel<true><<<grid, kAvgBins, 0, st>>>(P, S, n_used, idx, parts, squares, mean);
+        average_err_kernel<<<grid.x, kAvgBins, 0, st>>>(P, n_used, squares, err);
+        *launches += 6;
+    }
+    residual_of_kernel<<<P.n_tau_pad / 32, 32, 0, st>>>(P, mean, R_mean);
+    chi2_of_kernel<<<1, 128, 0, st>>>(P, R_mean, chi2_mean);
     return cudaGetLastError();
 }
 

@@ -184,9 +184,11 @@ cudaError_t launch_imprint_rows(const DevProblem &P, const DevState &S, int prec
 cudaError_t launch_smooth(const DevProblem &P, const DevState &S, int precision, double s, cudaStream_t st);
 cudaError_t launch_block_stats(const DevProblem &P, const DevState &S, BlockCounters *out,
                                cudaStream_t st);
+// idx: scratch of n_walkers; parts (FP32 state): scratch of 2 kAvgChunks n_omega.
+constexpr int kAvgChunks = 64;
 cudaError_t launch_average(const DevProblem &P, const DevState &S, int precision, double factor,
-                           double *mean, double *err, int *n_used, double *cut, double *R_mean,
-                           double *chi2_mean, cudaStream_t st, int *launches);
+                           double *mean, double *err, int *n_used, double *cut, int *idx, double *parts,
+                           double *R_mean, double *chi2_mean, cudaStream_t st, int *launches);
 cudaError_t launch_probe(const DevProblem &P, const DevState &S, int precision, int n,
                          const int *walker, const int *p, const int *s, const double *eps,
                          double *delta, int *ok, cudaStream_t st);
