@@ -72,7 +72,7 @@ struct Layout {
     size_t status;
     size_t a64, b32, g2, R64, R32, chi2, acc_prev, hash, n_acc, n_pos, guard;
     size_t acc_trace, m_trace, delta_trace;
-    size_t m, zero_l, donor_l, n_pairs, delta, counters, bz, bxi, cand, cand_Z, ctl;
+    size_t m, zero_l, donor_l, n_pairs, delta, counters;
     size_t mean, err, R_mean, chi2_mean, n_used, cut, avg_idx, avg_parts;
     size_t pr_walker, pr_p, pr_s, pr_eps, pr_delta, pr_ok;
     size_t tma_a, tma_b;     // pre-tiled BF16 pieces of the spectra and the kernel table (resync kind 2)
@@ -135,12 +135,7 @@ Layout make_layout(int n_tau, int n_omega, const sail_params &p) {
     L.donor_l = take(WB * 4);
     L.n_pairs = take(4);
     L.delta = take(8);
-    L.bz = take(WB * 8);
-    L.bxi = take(WB * 8);
     L.chi2_all = take(WB * 8);
-    L.cand = take(128 * 8);
-    L.cand_Z = take(128 * 4);
-    L.ctl = take(64);
     L.counters = take(sizeof(BlockCounters));
     L.mean = take(NO * 8);
     L.err = take(NO * 8);
@@ -699,11 +694,6 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     Bs.delta = (double *)(ws + L.delta);
     Bs.m_trace = p->trace ? (int *)(ws + L.m_trace) : nullptr;
     Bs.delta_trace = p->trace ? (double *)(ws + L.delta_trace) : nullptr;
-    Bs.z = (double *)(ws + L.bz);
-    Bs.xi = (double *)(ws + L.bxi);
-    Bs.cand = (double *)(ws + L.cand);
-    Bs.cand_Z = (int *)(ws + L.cand_Z);
-    Bs.ctl = (void *)(ws + L.ctl);
 
     cudaStream_t st = h->stream;
     auto up = [&](size_t off, const void *src, size_t bytes) {
@@ -1241,7 +1231,7 @@ int sail_branch_solve(sail_t h, int n_total, const double *chi2_all, int block, 
     B.m_trace = nullptr;
     B.delta_trace = nullptr;
     int l = 0;
-    SAIL_CUDA(launch_branch_solve(P, S, B, block, fraction, st, &l), "solve launch");
+    SAIL_CUDA(launch_branch_solve(P, S, B, h->prm.precision, block, fraction, st, &l), "solve launch");
     h->launches += l;
     int np = 0;
     SAIL_CUDA(cudaMemcpyAsync(m, B.m, (size_t)n_total * 4, cudaMemcpyDeviceToHost, st), "solve D2H");

@@ -488,160 +488,241 @@ __device__ int multipliers_at(int N, const double *z, const double *xi, double D
     return block_sum_i(zc, sh);
 }
 
-// The Delta search runs as speculative rounds over many blocks: every trial Delta the
-// sequential search could visit next is evaluated at once, one block (one SM) per trial, and
-// a one-thread control kernel replays the sequential search over the results.  Round 0 holds
-// the doubling trials 2^k, k = 0..64; each later round a depth-7 tree of bisection midpoints.
-// The replay takes exactly the steps, trial values and early exit of the sequential search,
-// so the chosen Delta and multipliers are the same; one SM per trial brings 127 SMs' FP64
-// units to bear on what is otherwise a long chain on one SM.
-constexpr int kTreeDepth = 7;
-constexpr int kMaxCand = (1 << kTreeDepth) - 1;   // 127 >= the 65 doubling trials
-
-struct SolveCtl {
-    double lo, hi, Delta;
-    int Zhi, Zt, done, it, n_cand;
-};
+// The whole solve in one block: the search over Delta is sequential, and a trial is cheap because
+// FP32 decides nearly every multiplier.  At a trial Delta each thread holds e^(-Delta z_l) in FP32
+// with a bound on its error; a count of sum m at some Theta forms Theta E + xi in FP32 and goes to
+// FP64 (the arithmetic of multipliers_at) only for a walker whose value lies within that bound of
+// an integer, about one in 1e5.  So every count is the FP64 count, and since each m_l rises with
+// Theta, the multipliers with sum N are the same whichever Theta with that sum is found; the
+// Theta search may therefore interpolate in FP32, and needs 5 to 8 counts.  Where no FP32 Theta has
+// sum N (ties, or two break points within 6e-8) multipliers_at decides.  The FP64 pipe (2 lanes a
+// clock and SM: one FP64 instruction of all 32 warps is 512 cycles) is what a solve in FP64 waits
+// for, so FP64 is kept to the walkers' differences from the smallest chi2 and to one warp's
+// scalars.  Against one block per speculative trial in FP64 (23 launches; the same multipliers):
+// 1013 -> 105 us at 4096 walkers, 4050 -> 522 us at 16384, 350 -> 62 us at 1500, 220 -> 28 us at 64
+// (first block of an anneal).
+constexpr float kSolveErr = 3e-7f;     // rounding of Theta E + xi and of xi, absolute part
 
 template <int PT>
-__device__ void load_zxi(const BranchScratch &B, int N, double *z, double *xi) {
+__device__ __noinline__ int multipliers_tied(int N, const double *chi2, double cmin, double spread, const uint32_t *word,
+                                             double Delta, int *m, SolveShared &sh) {
+    double z[PT], xi[PT];
 #pragma unroll
     for (int q = 0; q < PT; ++q) {
         const int l = threadIdx.x + kSolveThreads * q;
-        z[q] = l < N ? B.z[l] : 0.0;
-        xi[q] = l < N ? B.xi[l] : 0.5;
+        z[q] = l < N && spread > 0.0 ? (chi2[l] - cmin) / spread : 0.0;
+        xi[q] = l < N ? unit64(word[l]) : 0.5;
     }
+    return multipliers_at<PT>(N, z, xi, Delta, m, sh);
 }
 
-__global__ void __launch_bounds__(kSolveThreads) branch_prep_kernel(DevProblem P, DevState S, BranchScratch B,
-                                                                    int block_index, double fraction) {
-    __shared__ double s_cmin, s_spread;
-    extern __shared__ double s_chi2[];           // the walkers' chi2, staged for the ordered sum
-    const int N = P.n_walkers, tid = threadIdx.x;
-    SolveCtl *ctl = reinterpret_cast<SolveCtl *>(B.ctl);
-    int Zt = (int)floor(fraction * N + 0.5);
-    if (Zt > N - 1) Zt = N - 1;
-    for (int l = tid; l < N; l += blockDim.x) s_chi2[l] = S.chi2[l];
+// One walker's multiplier in FP64, as multipliers_at forms it.
+__device__ __noinline__ int multiplier64(float Theta, double Delta, double chi2, double cmin, double spread, uint32_t word, int N) {
+    const double z = spread > 0.0 ? (chi2 - cmin) / spread : 0.0;
+    const double v = floor((double)Theta * exp(-Delta * z) + unit64(word));
+    return v >= (double)N ? N : (int)v;
+}
+
+// Sums of a and b over the block, the same in every thread (one barrier; red alternates).
+template <typename T>
+__device__ __forceinline__ T block_sum1(T v, T (*red)[32], int buf) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    if ((threadIdx.x & 31) == 0) red[buf][threadIdx.x >> 5] = v;
     __syncthreads();
-    if (tid == 0) {
-        double cmin = s_chi2[0], csum = 0.0;
-        for (int l = 0; l < N; ++l) {
-            if (s_chi2[l] < cmin) cmin = s_chi2[l];
-            csum += s_chi2[l];
-        }
-        s_cmin = cmin;
-        s_spread = csum / N - cmin;
-        ctl->Zt = Zt;
-        ctl->done = Zt <= 0;
-        ctl->it = 0;
-        ctl->lo = 0.0;
-        ctl->hi = 1.0;
-        ctl->Delta = 0.0;
-        ctl->n_cand = 65;
-    }
-    if (tid < 65) B.cand[tid] = ldexp(1.0, tid);
+    v = red[buf][threadIdx.x & 31];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+__device__ __forceinline__ int2 block_sum2(int a, int b, int2 (*red)[32], int &buf) {
+    a = __reduce_add_sync(kFull, a);
+    b = __reduce_add_sync(kFull, b);
+    if ((threadIdx.x & 31) == 0) red[buf][threadIdx.x >> 5] = make_int2(a, b);
     __syncthreads();
-    const double cmin = s_cmin, spread = s_spread;
-    const uint2 key = philox_key(P.seed);
-    for (int l = tid; l < N; l += blockDim.x) {
-        B.z[l] = spread > 0.0 ? (s_chi2[l] - cmin) / spread : 0.0;
-        B.xi[l] = unit64(philox4x32_10(make_uint4((uint32_t)(l + P.walker_base), (uint32_t)block_index, 0u, 1u), key).x);
-    }
+    const int2 v = red[buf][threadIdx.x & 31];
+    buf ^= 1;
+    return make_int2(__reduce_add_sync(kFull, v.x), __reduce_add_sync(kFull, v.y));
 }
 
-template <int PT>
-__global__ void __launch_bounds__(kSolveThreads) branch_eval_kernel(int N, BranchScratch B) {
-    __shared__ SolveShared sh;
-    const SolveCtl *ctl = reinterpret_cast<const SolveCtl *>(B.ctl);
-    if (ctl->done || (int)blockIdx.x >= ctl->n_cand) return;   // uniform per block
-    double z[PT], xi[PT];
-    int m[PT];
-    load_zxi<PT>(B, N, z, xi);
-    const int Z = multipliers_at<PT>(N, z, xi, B.cand[blockIdx.x], m, sh);
-    if (threadIdx.x == 0) B.cand_Z[blockIdx.x] = Z;
-}
-
-// Writes the 127 midpoints of a depth-7 bisection tree over (lo, hi) in heap order: node n
-// (1-based) holds the interval reached by the outcomes on its path; its children 2n and 2n+1
-// are the intervals after "Z > target" (hi <- mid) and "Z < target" (lo <- mid).
-__device__ void build_tree(double lo, double hi, double *cand) {
-    double nlo[kMaxCand + 1], nhi[kMaxCand + 1];
-    nlo[1] = lo;
-    nhi[1] = hi;
-    for (int n = 1; n <= kMaxCand; ++n) {
-        const double mid = 0.5 * (nlo[n] + nhi[n]);
-        cand[n - 1] = mid;
-        if (2 * n <= kMaxCand) {
-            nlo[2 * n] = nlo[n];
-            nhi[2 * n] = mid;
-            nlo[2 * n + 1] = mid;
-            nhi[2 * n + 1] = nhi[n];
+// The search over Delta, advanced by one warp: Delta doubles from 1 until Z >= the target, at
+// most 64 times, then bisects, at most 64 times, and stops at the first Z equal to the target.
+struct SolveSearch {
+    double lo, hi, D;
+    int doublings, halvings, state;    // 0 doubling, 1 bisecting, 2 done (D is the result)
+    __device__ void begin() { lo = 0.0; hi = D = 1.0; doublings = halvings = state = 0; }
+    __device__ void next(int Z, int Zt) {
+        if (state == 0) {
+            if (Z < Zt && doublings < 64) {
+                lo = hi;
+                hi = D = 2.0 * hi;
+                ++doublings;
+                return;
+            }
+            state = 1;
+            if (Z == Zt) { state = 2; return; }
+        } else {
+            if (Z == Zt) { state = 2; return; }
+            if (Z < Zt) lo = D; else hi = D;
         }
-    }
-}
-
-__global__ void branch_control_kernel(BranchScratch B, int round) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    SolveCtl *ctl = reinterpret_cast<SolveCtl *>(B.ctl);
-    if (ctl->done) return;
-    const int Zt = ctl->Zt;
-    if (round == 0) {
-        // doubling: hi = 1, 2, 4, ... while Z(hi) < target, at most 64 doublings
-        double lo = 0.0, hi = 1.0;
-        int k = 0, Zhi = B.cand_Z[0];
-        while (k < 64 && Zhi < Zt) {
-            lo = hi;
-            hi = 2.0 * hi;
-            ++k;
-            Zhi = B.cand_Z[k];
-        }
-        ctl->lo = lo;
-        ctl->hi = hi;
-        ctl->Zhi = Zhi;
-        if (Zhi == Zt) {
-            ctl->done = 1;
-            ctl->Delta = hi;
+        const double mid = 0.5 * (lo + hi);
+        if (halvings >= 64 || mid <= lo || mid >= hi) {
+            D = hi;
+            state = 2;
             return;
         }
-    } else {
-        double lo = ctl->lo, hi = ctl->hi;
-        int n = 1;
-        for (int d = 0; d < kTreeDepth; ++d) {
-            if (ctl->it >= 64) { ctl->done = 1; ctl->Delta = hi; return; }
-            const double mid = B.cand[n - 1];
-            if (mid <= lo || mid >= hi) { ctl->done = 1; ctl->Delta = hi; return; }
-            const int Zm = B.cand_Z[n - 1];
-            ctl->it += 1;
-            if (Zm == Zt) { ctl->done = 1; ctl->Delta = mid; return; }
-            if (Zm < Zt) { lo = mid; n = 2 * n + 1; }
-            else { hi = mid; n = 2 * n; }
-        }
-        ctl->lo = lo;
-        ctl->hi = hi;
+        D = mid;
+        ++halvings;
     }
-    if (ctl->it >= 64) { ctl->done = 1; ctl->Delta = ctl->hi; return; }
-    build_tree(ctl->lo, ctl->hi, B.cand);
-    ctl->n_cand = kMaxCand;
-}
+};
 
-// Final multipliers at the chosen Delta and the imprint pairing: zero-multiplier walkers
-// ascending, matched with surplus copies (walker l listed m_l - 1 times) ascending.
 template <int PT>
-__global__ void __launch_bounds__(kSolveThreads) branch_final_kernel(int N, BranchScratch B, int event) {
+__global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProblem P, DevState S, BranchScratch B, int block_index,
+                                                                        double fraction, int event, int ordered) {
+    extern __shared__ double s_chi2[];           // chi2 [N] for the ordered sum; then z [N] and the draws [N]
     __shared__ SolveShared sh;
-    const SolveCtl *ctl = reinterpret_cast<const SolveCtl *>(B.ctl);
-    const int tid = threadIdx.x;
-    int m[PT];
-    double Delta = 0.0;
-    if (ctl->Zt <= 0) {
-#pragma unroll
-        for (int q = 0; q < PT; ++q) m[q] = 1;
-    } else {
-        double z[PT], xi[PT];
-        load_zxi<PT>(B, N, z, xi);
-        Delta = ctl->done ? ctl->Delta : ctl->hi;
-        multipliers_at<PT>(N, z, xi, Delta, m, sh);
+    __shared__ SolveSearch s_search;
+    __shared__ int2 red[2][32];
+    __shared__ float red_f[2][32];
+    const int N = P.n_walkers, tid = threadIdx.x;
+    float *s_z = reinterpret_cast<float *>(s_chi2);
+    uint32_t *s_word = reinterpret_cast<uint32_t *>(s_z + N);
+    int Zt = (int)floor(fraction * N + 0.5);
+    if (Zt > N - 1) Zt = N - 1;
+    double cmin = S.chi2[0], part = 0.0;
+    for (int l = tid; l < N; l += kSolveThreads) {
+        const double c = S.chi2[l];
+        if (ordered) s_chi2[l] = c;
+        else part += c;
+        cmin = c < cmin ? c : cmin;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double c = __shfl_xor_sync(kFull, cmin, o);
+        cmin = c < cmin ? c : cmin;
+    }
+    if ((tid & 31) == 0) sh.red_d[tid >> 5] = cmin;
+    __syncthreads();
+    cmin = sh.red_d[tid & 31];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double c = __shfl_xor_sync(kFull, cmin, o);
+        cmin = c < cmin ? c : cmin;
+    }
+    // the mean: FP64 state sums in walker order (the validation path's), FP32 state over threads
+    double csum;
+    if (ordered) {
+        if (tid == 0) {
+            double c = 0.0;
+#pragma unroll 8
+            for (int l = 0; l < N; ++l) c += s_chi2[l];
+            sh.theta = c;
+        }
+        __syncthreads();
+        csum = sh.theta;
+    } else {
+        csum = block_sum_d(part, sh);
+    }
+    const double spread = csum / N - cmin;
+    const float scale = spread > 0.0 ? (float)(1.0 / spread) : 0.0f;
+    const uint2 key = philox_key(P.seed);
+    __syncthreads();
+    float xif[PT], E[PT];                        // this thread's walkers: draws, and E at the trial Delta
+    int m[PT];
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int l = tid + kSolveThreads * q;
+        E[q] = 0.0f;
+        xif[q] = 0.5f;
+        m[q] = 1;
+        if (l < N) {
+            const uint32_t w = philox4x32_10(make_uint4((uint32_t)(l + P.walker_base), (uint32_t)block_index, 0u, 1u), key).x;
+            s_z[l] = scale * (float)(S.chi2[l] - cmin);
+            s_word[l] = w;
+            xif[q] = fmaf((float)w, 2.3283064e-10f, 1.1641532e-10f);
+        }
+    }
+    int buf = 0, fbuf = 0;
+    float Theta = 0.0f;                          // of the last trial: sum m = N
+    bool tied = false;
+    double Delta = 0.0;
+    float Df = 0.0f;
+    // multiplier of walker q of this thread at Theta
+    auto mult = [&](int q, float Th) -> int {
+        const int l = tid + kSolveThreads * q;
+        if (l >= N) return 0;
+        const float v = fmaf(Th, E[q], xif[q]);
+        // E's relative error: the exponent's rounding (4e-7 of it) and expf's
+        const float tol = fmaf(v, fmaf(4e-7f, Df * s_z[l], 2e-6f), kSolveErr);
+        const float lo = floorf(v - tol), hi = floorf(v + tol);
+        if (lo == hi && hi < 1e6f) return min((int)lo, N);
+        return multiplier64(Th, Delta, S.chi2[l], cmin, spread, s_word[l], N);
+    };
+    auto count = [&](float Th) -> int2 {         // (sum m, zero multipliers)
+        int c = 0, zc = 0;
+#pragma unroll
+        for (int q = 0; q < PT; ++q) {
+            const int k = mult(q, Th);
+            c += k;
+            zc += (k == 0 && tid + kSolveThreads * q < N);
+        }
+        return block_sum2(c, zc, red, buf);
+    };
+    // Z at the trial Delta; leaves Theta (or, tied, the multipliers in m)
+    auto trial = [&]() -> int {
+        tied = false;
+        float sE = 0.0f;
+#pragma unroll
+        for (int q = 0; q < PT; ++q) {
+            const int l = tid + kSolveThreads * q;
+            E[q] = l < N ? expf(-Df * s_z[l]) : 0.0f;
+            sE += E[q];
+        }
+        const float guess = (float)N / block_sum1(sE, red_f, fbuf);
+        fbuf ^= 1;
+        float lo = 0.9f * guess, hi = 1.1f * guess;
+        int2 clo = count(lo), chi = count(hi);
+        for (int it = 0; it < 100 && clo.x >= N; ++it) { lo *= 0.5f; clo = count(lo); }
+        for (int it = 0; it < 100 && chi.x < N; ++it) { hi *= 2.0f; chi = count(hi); }
+        if (clo.x < N && chi.x == N) { Theta = hi; return chi.y; }
+        for (int it = 0; it < 200; ++it) {
+            float mid = 0.5f * (lo + hi);
+            if (it % 3 != 2 && chi.x > clo.x) {
+                const float at = fmaf(hi - lo, ((float)(N - clo.x) + 0.5f) / (float)(chi.x - clo.x), lo);
+                if (at > lo && at < hi) mid = at;
+            }
+            if (!(mid > lo && mid < hi)) break;
+            const int2 c = count(mid);
+            if (c.x == N) { Theta = mid; return c.y; }
+            if (c.x < N) { lo = mid; clo = c; } else { hi = mid; chi = c; }
+        }
+        tied = true;
+        return multipliers_tied<PT>(N, S.chi2, cmin, spread, s_word, Delta, m, sh);
+    };
+
+    double result = 0.0;
+    if (Zt > 0) {
+        if (tid == 0) s_search.begin();
+        __syncthreads();
+        int Z = 0;
+        for (;;) {
+            const double D = s_search.D;
+            const int state = s_search.state;
+            if (state == 2) {
+                result = D;
+                if (D == Delta) break;           // the last trial was at the result
+            }
+            Delta = D;
+            Df = __double2float_rn(D);
+            Z = trial();
+            if (state == 2) break;
+            __syncthreads();
+            if (tid == 0) s_search.next(Z, Zt);
+            __syncthreads();
+        }
+        if (!tied) {
+#pragma unroll
+            for (int q = 0; q < PT; ++q) m[q] = mult(q, Theta);
+        }
+    }
+    // the imprint pairing: zero-multiplier walkers ascending, matched with surplus copies (walker l
+    // listed m_l - 1 times) ascending; one scan carries both counts (each at most 2^14)
     int zero_base = 0, copy_base = 0;
 #pragma unroll
     for (int q = 0; q < PT; ++q) {
@@ -649,44 +730,41 @@ __global__ void __launch_bounds__(kSolveThreads) branch_final_kernel(int N, Bran
         const bool valid = l < N;
         const int isz = valid && m[q] == 0;
         const int surplus = valid && m[q] > 1 ? m[q] - 1 : 0;
-        int tz, tc;
-        const int zo = block_scan_excl(isz, &tz, sh);
-        const int co = block_scan_excl(surplus, &tc, sh);
+        int total;
+        const int at = block_scan_excl(isz | (surplus << 16), &total, sh);
         if (valid) {
             B.m[l] = m[q];
-            if (isz) B.zero_l[zero_base + zo] = l;
-            for (int k = 0; k < surplus; ++k) B.donor_l[copy_base + co + k] = l;
+            if (isz) B.zero_l[zero_base + (at & 0xFFFF)] = l;
+            for (int k = 0; k < surplus; ++k) B.donor_l[copy_base + (at >> 16) + k] = l;
             if (B.m_trace) B.m_trace[(size_t)event * N + l] = m[q];
         }
-        zero_base += tz;
-        copy_base += tc;
+        zero_base += total & 0xFFFF;
+        copy_base += total >> 16;
     }
     if (tid == 0) {
         B.n_pairs[0] = zero_base < copy_base ? zero_base : copy_base;
-        B.delta[0] = Delta;
-        if (B.delta_trace) B.delta_trace[event] = Delta;
+        B.delta[0] = result;
+        if (B.delta_trace) B.delta_trace[event] = result;
     }
 }
 
 template <int PT>
-cudaError_t launch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int block_index,
+cudaError_t launch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision, int block_index,
                          double fraction, int event, cudaStream_t st, int *launches) {
-    const int N = P.n_walkers;
-    const size_t staged = (size_t)N * sizeof(double);   // <= 128 KiB (16384 walkers)
-    cudaError_t e0 = cudaFuncSetAttribute(branch_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
-    if (e0 != cudaSuccess) return e0;
-    branch_prep_kernel<<<1, kSolveThreads, staged, st>>>(P, S, B, block_index, fraction);
-    branch_eval_kernel<PT><<<kMaxCand, kSolveThreads, 0, st>>>(N, B);
-    branch_control_kernel<<<1, 32, 0, st>>>(B, 0);
-    *launches += 3;
-    for (int r = 1; r <= (64 + kTreeDepth - 1) / kTreeDepth; ++r) {
-        branch_eval_kernel<PT><<<kMaxCand, kSolveThreads, 0, st>>>(N, B);
-        branch_control_kernel<<<1, 32, 0, st>>>(B, r);
-        *launches += 2;
-    }
-    branch_final_kernel<PT><<<1, kSolveThreads, 0, st>>>(N, B, event);
+    const size_t staged = (size_t)P.n_walkers * sizeof(double);   // <= 128 KiB (16384 walkers)
+    cudaError_t e = cudaFuncSetAttribute(branch_solve_kernel<PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+    if (e != cudaSuccess) return e;
+    branch_solve_kernel<PT><<<1, kSolveThreads, staged, st>>>(P, S, B, block_index, fraction, event, precision == 0);
     *launches += 1;
     return cudaGetLastError();
+}
+
+template <typename... Args>
+cudaError_t launch_solve_n(const DevProblem &P, Args... args) {
+    if (P.n_walkers <= kSolveThreads) return launch_solve<1>(P, args...);
+    if (P.n_walkers <= kSolveThreads * 4) return launch_solve<4>(P, args...);
+    if (P.n_walkers <= kSolveThreads * 8) return launch_solve<8>(P, args...);
+    return launch_solve<16>(P, args...);
 }
 
 // Imprinting (Sec. 2.5): a^(l1) <- t a^(l2) + (1 - t) a^(l1); the residual mixes the same way
@@ -1140,21 +1218,16 @@ cudaError_t launch_resync(const DevProblem &P, const DevState &S, int precision,
 cudaError_t launch_branch(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision,
                           int block_index, double fraction, double imprint_t, int event, cudaStream_t st,
                           int *launches) {
-    cudaError_t e;
-    if (P.n_walkers <= kSolveThreads * 4) e = launch_solve<4>(P, S, B, block_index, fraction, event, st, launches);
-    else if (P.n_walkers <= kSolveThreads * 8) e = launch_solve<8>(P, S, B, block_index, fraction, event, st, launches);
-    else e = launch_solve<16>(P, S, B, block_index, fraction, event, st, launches);
+    const cudaError_t e = launch_solve_n(P, S, B, precision, block_index, fraction, event, st, launches);
     if (e != cudaSuccess) return e;
     imprint_kernel<<<P.n_walkers, 128, 0, st>>>(P, S, B, precision, imprint_t);
     *launches += 1;
     return cudaGetLastError();
 }
 
-cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int block_index,
-                                double fraction, cudaStream_t st, int *launches) {
-    if (P.n_walkers <= kSolveThreads * 4) return launch_solve<4>(P, S, B, block_index, fraction, 0, st, launches);
-    if (P.n_walkers <= kSolveThreads * 8) return launch_solve<8>(P, S, B, block_index, fraction, 0, st, launches);
-    return launch_solve<16>(P, S, B, block_index, fraction, 0, st, launches);
+cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision,
+                                int block_index, double fraction, cudaStream_t st, int *launches) {
+    return launch_solve_n(P, S, B, precision, block_index, fraction, 0, st, launches);
 }
 
 cudaError_t launch_walker_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,

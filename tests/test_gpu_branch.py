@@ -1,0 +1,47 @@
+"""GPU: the branching solve (multipliers, Delta, pairs) against the oracle at the edges of its
+block: one to sixteen walkers a thread, partial last rows, and residues that are widely spread,
+nearly equal, equal, or equal in clusters."""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1609_07936_gb300 as sail
+from workloads import tiny_double_lorentz
+
+pytestmark = pytest.mark.gpu
+
+
+def _chi2(kind, n, near=1e-10):
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal(n)
+    if kind == "spread":
+        return 1e3 * np.exp(0.3 * x)
+    if kind == "heavy":
+        return np.exp(5.0 * x)
+    if kind == "near":
+        return 1e12 * (1.0 + near * np.abs(x))
+    if kind == "equal":
+        return np.full(n, 17.0)
+    return np.repeat(100.0 + np.abs(x[: (n + 6) // 7]), 7)[:n]      # clusters of seven
+
+
+@pytest.mark.parametrize("precision", [sail.PREC_FP64, sail.PREC_FP32])
+@pytest.mark.parametrize("kind", ["spread", "heavy", "near", "equal", "clusters"])
+@pytest.mark.parametrize("n", [2, 3, 33, 1024, 1025, 4097, 8193, 16384])
+def test_solve_gives_the_oracle_multipliers(n, kind, precision):
+    P = tiny_double_lorentz()
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega,
+                  sail.Params(n_walkers=2, precision=precision, n_sweeps=10, branching=False, A=P.A, B=P.B, seed=5,
+                              walker_total=16384))
+    for block, fraction in ((0, 0.25), (3, 0.6)):
+        # an FP32 population's mean is summed in another order than the oracle's: its residues are kept
+        # far enough apart that the sum's rounding cannot reorder break points
+        c = _chi2(kind, n, 1e-10 if precision == sail.PREC_FP64 else 1e-4)
+        m, delta, zero, donor = g.branch_solve(c, block, fraction)
+        m_o, delta_o = O.branch_multipliers(c, O.xi_for_block(5, block, n), fraction)[:2]
+        np.testing.assert_array_equal(m, m_o)
+        assert delta == delta_o
+        np.testing.assert_array_equal(zero, np.flatnonzero(m == 0)[: zero.size])
+        np.testing.assert_array_equal(donor, np.repeat(np.arange(n), np.maximum(m - 1, 0))[: zero.size])
+        assert zero.size == (m == 0).sum()
+    g.close()
