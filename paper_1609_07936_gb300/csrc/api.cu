@@ -1427,7 +1427,6 @@ struct sail_batch_ctx {
     // lanes per walker (16 or 8), or the span sweep, times move-loop variant (plain, walk,
     // Hastings); class = 3 * (lanes == 8) + mode, or 6 + mode for the span sweep
     static constexpr int kClasses = 9;
-    int span_lanes;            // lanes per walker of the plain span class in this segment (4 or 8)
     size_t smem[kClasses];     // shared memory of each class's kernel: its problems' largest tables
     cudaStream_t aux[kClasses - 1];   // further streams: the classes' kernels run side by side
     cudaEvent_t fork, join[kClasses - 1];
@@ -1523,7 +1522,7 @@ cudaError_t batch_sweep_segment(sail_batch_ctx *b, const int *count) {
         cudaStream_t sc = k == 0 ? st : b->aux[k - 1];
         if (c >= 6)
             e = launch_span_batch(b->d_probs, b->d_items + offset, count[c], b->d_counter + c, b->smem[c], b->item_pairs,
-                                  b->span_lanes, c - 6, sc);
+                                  c - 6, sc);
         else
             e = launch_sweep_batch(b->d_probs, b->d_items + offset, count[c], b->d_counter + c, b->smem[c], b->item_pairs,
                                    c >= 3 ? 8 : 16, c % 3, sc);
@@ -1671,11 +1670,7 @@ int batch_run_blocks(sail_batch_ctx *b, int max_blocks, int *n_done) {
         for (;;) {
             // one segment: every problem with sweeps left in this block advances to its next resync
             for (auto &v : cls_items) v.clear();
-            long long seg_moves = 0, span_walkers = 0;
-            for (int k = 0; k < N; ++k)
-                if (active[k] && cur[k] < pend[k].block_end && batch_class(b->h[k]->P) == 6)
-                    span_walkers += b->h[k]->prm.n_walkers;
-            b->span_lanes = span_batch_lanes(span_walkers);
+            long long seg_moves = 0;
             for (int k = 0; k < N; ++k) {
                 sail_ctx *h = b->h[k];
                 hp[k].n0 = hp[k].n1 = 0;
@@ -1686,7 +1681,7 @@ int batch_run_blocks(sail_batch_ctx *b, int max_blocks, int *n_done) {
                 hp[k].n1 = next_resync(h, cur[k], pend[k].block_end);
                 seg_moves += (long long)(hp[k].n1 - hp[k].n0) * h->prm.n_walkers * h->n_omega;
                 const int cls = batch_class(h->P);
-                const int wpw = cls >= 6 ? 32 / (cls == 6 ? b->span_lanes : 8) : sweep_walkers_per_warp(h->P);
+                const int wpw = cls >= 6 ? 32 / span_batch_lanes(cls - 6) : sweep_walkers_per_warp(h->P);
                 const int groups = (h->prm.n_walkers + wpw - 1) / wpw;
                 // walker groups per item = warps per block (over tau at most 8 with 8 lanes per walker,
                 // 12 with 16; span sweep 16)

@@ -213,12 +213,12 @@ cudaError_t launch_sweep_batch(const BatchProblem *d_probs, const BatchItem *d_i
 cudaError_t launch_sweep_batch8(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                 size_t smem, int warps, int mode, cudaStream_t st);
 // The batched span sweep of problems whose P.span_on is set (any widths together): blocks of `warps`
-// warps (at most 16), lanes (4 or 8) per walker for the plain mode (8 for the others; the results do
-// not depend on it), smem at least the problems' span_batch_smem.
+// warps (at most 16), smem at least the problems' span_batch_smem; lanes per walker by mode (the
+// results do not depend on it).
 size_t span_batch_smem(const DevProblem &P, int smem_max);
-int span_batch_lanes(long long walkers);
+inline int span_batch_lanes(int mode) { return mode == 0 ? 4 : 8; }
 cudaError_t launch_span_batch(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
-                              size_t smem, int warps, int lanes, int mode, cudaStream_t st);
+                              size_t smem, int warps, int mode, cudaStream_t st);
 cudaError_t launch_read_probe(const void *buf, size_t bytes, int reps, void *sink, cudaStream_t st);
 cudaError_t launch_smem_probe(int reps, void *sink, cudaStream_t st, double *bytes);
 

@@ -10,7 +10,7 @@
 // the same number up to rounding: the part of R outside the span is constant and drops out.
 // A move costs RR elements instead of n_tau, and its two columns are two rows of a table that
 // fits in shared memory whole (96 KB at 1000 bins), not products of factor rows.  The residual
-// itself is not written back: every sweep launch is followed by its recomputation.
+// and chi2 are not written back: every sweep launch is followed by their recomputation.
 //
 // Rounding.  Fewer elements average out less rounding error, so three things keep the error of
 // delta chi2 below that of the loops over tau (measured in FP32 emulation against FP64 on the
@@ -23,10 +23,11 @@
 // carried along (Kahan), so it does not drift either.
 //
 // Measured against the loops over tau (sweep_group.cuh), sweep time, same box: 200 tau x 1000 bins
-// x 4096 walkers, 100 sweeps 47.1 -> 18.6 ms (2.2e10 walker-moves/s; 111 warp instructions an
-// iteration of four walkers, 382 cycles at 1.75 warps a scheduler: latency-bound), 16384 walkers
-// 198 -> 53 ms; 512 x 2048 x 16384, 10 sweeps 90 -> 14 ms; 160 x 1000 x 1500, 100 sweeps 35.5 ->
-// 14.8 ms; Hastings 72 -> 20 ms; index walk (1500 walkers, 50 sweeps) 47 -> 32 ms.
+// x 4096 walkers, 100 sweeps 47.1 -> 14.0 ms (2.9e10 walker-moves/s; 100 warp instructions an
+// iteration of four walkers, 290 cycles at two warps on a scheduler, 64% of its issue slots and 67%
+// of the shared-memory data pipe), 16384 walkers 198 -> 45 ms; 512 x 2048 x 16384, 10 sweeps 90 ->
+// 14 ms (spectra in L2); 160 x 1000 x 1500, 100 sweeps 35.5 -> 9.6 ms (203 cycles an iteration,
+// one warp); Hastings 72 -> 15.7 ms; index walk (1500 walkers, 50 sweeps) 47 -> 30 ms.
 //
 // Layout.  G lanes per walker (8 or 4: four or eight walkers a warp).  The RR elements belong to
 // eight virtual lanes, RR / 8 each; delta chi2 is the xor-butterfly sum (4, 2, 1) of the virtual
@@ -39,6 +40,13 @@
 // words and columns are read while move k is reduced, the amplitudes that move k would set are
 // formed before its test, and its update is branch-free.  The words of G consecutive moves are
 // drawn at once, one move per lane, and handed over through a ring in shared memory.
+//
+// One basic block.  The G moves of a batch are unrolled without a branch (stores under a predicate,
+// masked updates, a reciprocal without its slow path, null moves past the sweep's end), so that the
+// compiler fills a move's butterfly with the work around it: the same loop with branches for the
+// accepted move and the division ran 310 cycles an iteration instead of 203 (one warp), 387 instead
+// of 290 (4096 walkers).  Evaluating two moves at once (the second for both outcomes of the first)
+// halves the butterflies but costs 128 instructions a move: 2.28 against 1.98 ms.
 #pragma once
 #include "sweep_group.cuh"
 
@@ -207,23 +215,30 @@ __device__ __forceinline__ void span_d(const SpanVec<RR> (&g)[NV], const SpanVec
     }
 }
 
-// 1 / g, correctly rounded; g is a product of factors 1 - eps and stays far inside FP32's normal
-// range, so the subnormal cases (flushed here) do not occur.
+// 1 / g, correctly rounded, for g and 1 / g in FP32's normal range (g is a product of factors
+// 1 - eps over one launch): one Newton step y + y (1 - g y) in fused arithmetic from the hardware's
+// approximation (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990).  Equal to 1.0f / g for all 2^23 significands at every exponent from 2^-125 to
+// 2^125 (checked on the GPU).
 __device__ __forceinline__ float rcp_rn(float g) {
-    float r;
-    asm("rcp.rn.ftz.f32 %0, %1;" : "=f"(r) : "f"(g));
-    return r;
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(g));
+    return fmaf(y, fmaf(-g, y, 1.0f), y);
 }
 
-// b[j] = v if acc
+// b[p] = vp and b[s] = vs if take != 0
 template <bool SMEM>
-__device__ __forceinline__ void put_if(bool acc, float *b, int j, float v) {
+__device__ __forceinline__ void put_if(float take, float *b, int p, int s, float vp, float vs) {
     if constexpr (SMEM)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %0, 0;\n\t@p st.shared.f32 [%1], %2;\n\t}"
-                     ::"r"((int)acc), "r"((uint32_t)__cvta_generic_to_shared(b + j)), "f"(v) : "memory");
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.shared.f32 [%1], %3;\n\t"
+                     "@q st.shared.f32 [%2], %4;\n\t}"
+                     ::"f"(take), "r"((uint32_t)__cvta_generic_to_shared(b + p)),
+                     "r"((uint32_t)__cvta_generic_to_shared(b + s)), "f"(vp), "f"(vs) : "memory");
     else
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %0, 0;\n\t@p st.global.f32 [%1], %2;\n\t}"
-                     ::"r"((int)acc), "l"(__cvta_generic_to_global(b + j)), "f"(v) : "memory");
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.global.f32 [%1], %3;\n\t"
+                     "@q st.global.f32 [%2], %4;\n\t}"
+                     ::"f"(take), "l"(__cvta_generic_to_global(b + p)), "l"(__cvta_generic_to_global(b + s)), "f"(vp),
+                     "f"(vs) : "memory");
 }
 
 // The line of b[j] (global memory) into L1.
@@ -231,12 +246,69 @@ __device__ __forceinline__ void touch(const float *b, int j) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(b + j)));
 }
 
+// Lane's draw of move mv of walker wr.  The Metropolis test is D < threshold: D <= 0 passes, so a
+// plain threshold is at least the smallest positive float (the Hastings threshold may be negative).
+// Past the sweep's end, and for walkers that do not exist, a null move: eps = 1 makes its
+// amplitudes 0, which passes the positivity test (it is not counted), and the threshold is never met.
+template <int MODE>
+__device__ __forceinline__ MoveDraw span_draw(const DevProblem &P, int mv, int n, int wr, bool active, uint2 key, float yd,
+                                              float T, const float *sBeta, const float *sRgap) {
+    MoveDraw m = draw_move<MODE>(mv, n, wr + P.walker_base, key, P.n_omega, yd, T, sBeta, sRgap);
+    if constexpr (MODE != kHastings) m.thr = fmaxf(m.thr, 1.401298464e-45f);
+    if (mv >= P.n_omega || !active) {
+        m.eps = 1.0f;
+        m.dp = m.ds = 0.0f;
+        m.thr = -INFINITY;
+    }
+    return m;
+}
+__device__ __forceinline__ void span_put(SpanRing &ring, int batch, const MoveDraw &m) {
+    const int lane = threadIdx.x & 31;
+    ring.a[batch][lane] = make_float4(-m.dp, -m.dp, -m.ds, -m.ds);
+    ring.b[batch][lane] = make_float4(-m.eps, -m.eps, m.thr, __int_as_float(m.ps));
+}
+// Move i of the batch of this lane's walker.
+template <int G>
+__device__ __forceinline__ SpanMove span_get(const SpanRing &ring, int batch, int i) {
+    const int at = (threadIdx.x & 31) / G * G + i;
+    const float4 x = ring.a[batch][at], y = ring.b[batch][at];
+    SpanMove m;
+    m.mdp2 = pk(x.x, x.y);
+    m.mds2 = pk(x.z, x.w);
+    m.me2 = pk(y.x, y.y);
+    m.mdp = x.x;
+    m.mds = x.z;
+    m.me = y.x;
+    m.thr = y.z;
+    m.ps = __float_as_int(y.w);
+    return m;
+}
+
+// Folds the common scale into walker w's spectrum b and writes the walker back (lane gl of its G).
+template <int G>
+__device__ __forceinline__ void span_write_back(const DevProblem &P, const DevState &S, int w, int gl, const float *b, float ghi,
+                                                float glo, int accp, unsigned long long nacc,
+                                                unsigned long long npos) {
+    float *bg = S.b32 + (size_t)w * P.n_omega;
+    for (int j = gl; j < P.n_omega; j += G) {
+        const float v = b[j];
+        bg[j] = fmaf(glo, v, ghi * v);
+    }
+    if (gl == 0) {
+        S.g2[2 * w] = 1.0f;
+        S.g2[2 * w + 1] = 0.0f;
+        S.acc_prev[w] = accp;
+        S.n_acc[w] += nacc;
+        S.n_pos[w] += npos;
+    }
+}
+
 // Sweeps [n0, n1) for the 32 / G walkers of group grp of one problem on one warp.
 //   tab    the column table (shared memory if TS, else global memory), rows of RR floats
 //   sBeta, sRgap  beta and the reciprocal gaps (shared memory)
 //   b      STAGED: the spectra of walkers walker_lo.. in shared memory; else in global memory,
 //          where a move's b_p, b_s are read one move ahead (and patched if the move before it
-//          writes one of those bins): the read's latency is then off the chain
+//          writes one of those bins), from lines fetched into L1 a move earlier still
 // Every lane of a walker writes an accepted move's two amplitudes (the same values), so each
 // lane later reads its own write and the loop needs no barrier.
 template <int RR, int G, bool TS, bool STAGED, int MODE>
@@ -268,50 +340,18 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
     V R[NV], C[NV], F[NV];
     span_project<RR, NV>(P, S.R32 + (size_t)wr * P.n_tau_pad, vl, R, C, F);
     float ghi = S.g2[2 * wr], glo = S.g2[2 * wr + 1];
-    double chi2 = S.chi2[wr];
     int accp = S.acc_prev[wr];
     unsigned long long nacc = 0, npos = 0;
     const f2 two = pk(2.0f, 2.0f), minus_one = pk(-1.0f, -1.0f);
-
-    // Draws move mv into the ring.  The Metropolis test is D < threshold: D <= 0 passes, so a plain
-    // threshold is at least the smallest positive float (the Hastings threshold may be negative).
-    // Past the sweep's end, and for walkers that do not exist, a null move that is never accepted.
-    auto draw = [&](int mv, int n, float yd, float T) -> MoveDraw {
-        MoveDraw m = draw_move<MODE>(mv, n, wr + P.walker_base, key, NO, yd, T, sBeta, sRgap);
-        if constexpr (MODE != kHastings) m.thr = fmaxf(m.thr, 1.401298464e-45f);
-        if (mv >= NO || !active) {
-            m.eps = m.dp = m.ds = 0.0f;
-            m.thr = -INFINITY;
-        }
-        return m;
-    };
-    auto put = [&](int batch, const MoveDraw &m) {
-        ring.a[batch][lane] = make_float4(-m.dp, -m.dp, -m.ds, -m.ds);
-        ring.b[batch][lane] = make_float4(-m.eps, -m.eps, m.thr, __int_as_float(m.ps));
-    };
-    auto get = [&](int batch, int i) -> SpanMove {
-        const float4 x = ring.a[batch][sub * G + i], y = ring.b[batch][sub * G + i];
-        SpanMove m;
-        m.mdp2 = pk(x.x, x.y);
-        m.mds2 = pk(x.z, x.w);
-        m.me2 = pk(y.x, y.y);
-        m.mdp = x.x;
-        m.mds = x.z;
-        m.me = y.x;
-        m.thr = y.z;
-        m.ps = __float_as_int(y.w);
-        return m;
-    };
 
     for (int n = n0; n < n1; ++n) {
         const float T = (float)P.Tsweep[n];
         const float yd = (float)(amplitude(accp, NO, P.y_p, P.y_m, P.y_min) * dmove);
         int acc = 0, pos = 0;
-        float dchi = 0.0f;
         __syncwarp();
-        put(0, draw(gl, n, yd, T));
+        span_put(ring, 0, span_draw<MODE>(P, gl, n, wr, active, key, yd, T, sBeta, sRgap));
         __syncwarp();
-        SpanMove cur = get(0, 0), nxt = get(0, 1);
+        SpanMove cur = span_get<G>(ring, 0, 0), nxt = span_get<G>(ring, 0, 1);
         V g[NV];
         if constexpr (!WALK) span_g<RR, NV, TS>(tab, vl, F, cur, g);
         float bpc = 0.0f, bsc = 0.0f;          // BAHEAD: b at the current move's bins
@@ -321,12 +361,11 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
         }
         int batch = 0;
         for (int base = 0; base < NO; base += G, batch ^= 1) {
-            const MoveDraw mine = draw(base + G + gl, n, yd, T);    // the next G moves, one per lane
-            const int m_end = NO - base;
+            const MoveDraw mine = span_draw<MODE>(P, base + G + gl, n, wr, active, key, yd, T, sBeta, sRgap);
 #pragma unroll
             for (int i = 0; i < G; ++i) {
                 if (i == (G > 4 ? G - 3 : 1)) {
-                    put(batch ^ 1, mine);
+                    span_put(ring, batch ^ 1, mine);
                     __syncwarp();
                 }
                 if constexpr (WALK) {
@@ -388,7 +427,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                     bs = b[s];
                 }
                 if constexpr (!WALK) span_g<RR, NV, TS>(tab, vl, F, nxt, g);
-                const SpanMove far = i < G - 2 ? get(batch, i + 2) : get(batch ^ 1, i + 2 - G);
+                const SpanMove far = i < G - 2 ? span_get<G>(ring, batch, i + 2) : span_get<G>(ring, batch ^ 1, i + 2 - G);
                 if constexpr (BAHEAD) {
                     touch(b, far.ps & 0xFFFF);
                     touch(b, far.ps >> 16);
@@ -399,7 +438,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 const float ap = fmaf(r, ghi * bp, -cur.mdp);
                 const float as = fmaf(r, ghi * bs, -cur.mds);
                 const bool ok = ap >= 0.0f && as >= 0.0f;
-                pos += !ok && i < m_end;
+                pos += !ok;
                 float gah = ghi, gal = glo;
                 pair_scale(gah, gal, r);
                 const float inv_g = rcp_rn(gah);
@@ -411,9 +450,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 const f2 am2 = pk(am, am);
 #pragma unroll
                 for (int u = 0; u < NV; ++u) span_add<RR>(R[u], C[u], d[u], am, am2, minus_one);
-                put_if<STAGED>(acc_k, b, p, ap_b);
-                put_if<STAGED>(acc_k, b, s, as_b);
-                dchi += acc_k ? D : 0.0f;
+                put_if<STAGED>(am, b, p, s, ap_b, as_b);
                 ghi = acc_k ? gah : ghi;
                 glo = acc_k ? gal : glo;
                 acc += acc_k;
@@ -426,7 +463,6 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 nxt = far;
             }
         }
-        chi2 += (double)dchi;
         accp = acc;
         nacc += acc;
         npos += pos;
@@ -434,20 +470,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
     }
     __syncwarp();                      // the lanes' writes of b, before other lanes fold them
     if (!active) return;
-    // fold the common scale into the spectrum and write the walker back
-    float *bg = S.b32 + (size_t)w * NO;
-    for (int j = gl; j < NO; j += G) {
-        const float v = b[j];
-        bg[j] = fmaf(glo, v, ghi * v);
-    }
-    if (gl == 0) {
-        S.g2[2 * w] = 1.0f;
-        S.g2[2 * w + 1] = 0.0f;
-        S.chi2[w] = chi2;
-        S.acc_prev[w] = accp;
-        S.n_acc[w] += nacc;
-        S.n_pos[w] += npos;
-    }
+    span_write_back<G>(P, S, w, gl, b, ghi, glo, accp, nacc, npos);
 }
 
 // Shared memory of a span launch: rings, beta, gaps, then the table and the spectra if staged.
@@ -512,9 +535,9 @@ SpanGeom span_geom(const DevProblem &P, int sms, int smem_max, size_t *smem) {
     const int ctas = Gm.groups_total < sms ? Gm.groups_total : sms;
     Gm.groups_per_cta = (Gm.groups_total + ctas - 1) / ctas;
     Gm.rounds = (Gm.groups_per_cta + kSpanWarps - 1) / kSpanWarps;
+    const size_t tab = (size_t)P.n_omega * RR * 4, spec = (size_t)WPW * Gm.groups_per_cta * P.n_omega * 4;
     Gm.warps = (Gm.groups_per_cta + Gm.rounds - 1) / Gm.rounds;
     *smem = span_ring_bytes(Gm.warps) + (size_t)span_vec_floats(P.n_omega) * 4;
-    const size_t tab = (size_t)P.n_omega * RR * 4, spec = (size_t)WPW * Gm.groups_per_cta * P.n_omega * 4;
     Gm.stage_t = *smem + tab <= (size_t)smem_max;
     *smem += Gm.stage_t ? tab : 0;
     Gm.stage_b = Gm.stage_t && *smem + spec <= (size_t)smem_max;
@@ -533,11 +556,13 @@ cudaError_t launch_span_g(const DevProblem &P, const DevState &S, int n0, int n1
 }
 
 // Lanes per walker of a launch (either gives the same trajectories).  8 lanes keep one warp's chain
-// shortest and serve up to 64 walkers an SM at once.  4 lanes need 0.78 of the instructions per
-// walker: they run where 8 lanes would take a second round (16384 walkers, 200 x 1000: 10.7 ms
-// against 16.0 ms for 20 sweeps; 8192: 9.2 against 8.1), and where the population fills the
-// schedulers and its spectra fit in shared memory (4096 walkers, 32 x 64: 2.43 against 2.61 ms for
-// 200 sweeps; 608: 2.37 against 2.12).
+// shortest: they run while the spectra are staged and the SM's schedulers have room (20 sweeps, 200
+// x 1000: 1500 walkers 1.98 ms against 2.79 with 4 lanes, 4096: 2.81 against 5.7, which does not
+// stage).  4 lanes need 0.8 of the instructions per walker: they run where the spectra stay in
+// global memory anyway (8192 walkers 6.3 against 7.9 ms, 16384: 9.0 against 15.6; 512 x 2048: 608
+// walkers 11.2 against 14.9, 8192: 13.2 against 19.0), and where the population fills the
+// schedulers and is staged (32 x 64, 200 sweeps: 4096 walkers 1.67 against 1.86 ms; 608: 1.63
+// against 1.36).
 template <int RR, int MODE>
 cudaError_t launch_span(const DevProblem &P, const DevState &S, int n0, int n1, cudaStream_t st) {
     int dev = 0, sms = 0, smem_max = 0;
@@ -550,7 +575,7 @@ cudaError_t launch_span(const DevProblem &P, const DevState &S, int n0, int n1, 
     if constexpr (MODE != kWalk) {
         size_t m4 = 0;
         const SpanGeom g4 = span_geom<RR, 4>(P, sms, smem_max, &m4);
-        if (m4 <= (size_t)smem_max && (g8.rounds > 1 || (g4.stage_b && g8.groups_per_cta >= 6)))
+        if (m4 <= (size_t)smem_max && (!g8.stage_b || (g4.stage_b && g8.groups_per_cta >= 6)))
             return launch_span_g<RR, 4, MODE>(P, S, n0, n1, g4, m4, st);
     }
     return launch_span_g<RR, 8, MODE>(P, S, n0, n1, g8, m8, st);
