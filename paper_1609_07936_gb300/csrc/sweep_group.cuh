@@ -200,6 +200,32 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
     return d;
 }
 
+// 1 / g, correctly rounded, for g and 1 / g in FP32's normal range (g is a product of factors
+// 1 - eps over one launch): one Newton step y + y (1 - g y) in fused arithmetic from the hardware's
+// approximation (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990).  Equal to 1.0f / g for all 2^23 significands at every exponent from 2^-125 to
+// 2^125 (checked on the GPU).
+__device__ __forceinline__ float rcp_rn(float g) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(g));
+    return fmaf(y, fmaf(-g, y, 1.0f), y);
+}
+
+// b[p] = vp and b[s] = vs if take != 0
+template <bool SMEM>
+__device__ __forceinline__ void put_if(float take, float *b, int p, int s, float vp, float vs) {
+    if constexpr (SMEM)
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.shared.f32 [%1], %3;\n\t"
+                     "@q st.shared.f32 [%2], %4;\n\t}"
+                     ::"f"(take), "r"((uint32_t)__cvta_generic_to_shared(b + p)),
+                     "r"((uint32_t)__cvta_generic_to_shared(b + s)), "f"(vp), "f"(vs) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.global.f32 [%1], %3;\n\t"
+                     "@q st.global.f32 [%2], %4;\n\t}"
+                     ::"f"(take), "l"(__cvta_generic_to_global(b + p)), "l"(__cvta_generic_to_global(b + s)), "f"(vp),
+                     "f"(vs) : "memory");
+}
+
 // One chunk of the four factor rows a move needs (Qhi and Qlo rows of bins p and s): a lane's
 // E-float piece of each (shared-window addresses).
 __device__ __forceinline__ void ld_chunk(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, f2 (&v0)[1],
@@ -510,6 +536,13 @@ __device__ __forceinline__ bool guarded_accept(bool live, float &D, float S, flo
 // those whose move then fails the positivity test: with few warps per SM the sweep is bound by
 // the latency of each warp's instruction stream more than by shared-memory bandwidth.
 //
+// The G moves of a batch are one basic block (8 lanes; 4 of the 16 moves with 16 lanes): the update
+// is masked, the stores are predicated, the reciprocal has no slow path and a move past the sweep's
+// end is not live, so the compiler overlaps a move's butterfly and update with the next one's work.
+// Against the loop with branches, same box, 20 sweeps: 200 tau x 1000 bins x 4096 walkers 9.79 ->
+// 8.71 ms, 160 x 1000 x 1500 7.20 -> 4.61, Hastings 10.14 -> 9.05, index walk 22.6 -> 18.1 (one move
+// a block), 512 x 2048 x 16384 (4 sweeps) 35.0 -> 33.9; eight moves a block with 16 lanes: 36.3.
+//
 // BA (uniform bins only): each move's b_p, b_s are read one move ahead, during the move before
 // it, and patched if that move wrote one of those bins.  The batched kernel's plain loop, whose
 // spectra stay in global memory, takes this (measured +6% on uneven batches); the
@@ -528,6 +561,7 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
     constexpr bool WALK = MODE == kWalk;
     constexpr bool PIPE = C <= 8 && !WALK;
     constexpr bool BAHEAD = BA && !WALK;   // b read one move ahead (above)
+    constexpr int UNROLL = G == 8 ? 8 : 4;   // moves per basic block (see above)
     const int NO = P.n_omega, PAD = P.n_tau_pad;
     constexpr bool CT = G == 8;       // quad-compact tables with 8 lanes per walker
     const TabLayout TL = tab_layout(CT, NO, PAD);
@@ -595,138 +629,143 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
             bpc = bget(cur.ps & 0xFFFF);
             bsc = bget(cur.ps >> 16);
         }
-        for (int mv = 0; mv < NO; ++mv) {
-            if constexpr (WALK) {
-                // the index walk (Sec. 2.3) on the spectrum as it is now: lane t of the group
-                // draws step t + 1's words (counter (mv, n, w, 2 + t)), lane L the admixture's
-                const int L = P.walk_len;
-                const uint4 wr4 = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)(wr + P.walker_base), 2u + gl), key);
-                const bool walk_p = !(unit32(__shfl_sync(kFull, wr4.x, L, G)) < rho);
-                const bool walk_s = !(unit32(__shfl_sync(kFull, wr4.y, L, G)) < rho);
-                int wp = cur.ps & 0xFFFF;
-                float bp = bget(wp);
-                for (int t = 0; t < L; ++t) {
-                    const uint32_t xj = __shfl_sync(kFull, wr4.x, t, G), xu = __shfl_sync(kFull, wr4.y, t, G);
-                    const int j = (int)(((uint64_t)xj * (uint64_t)NO) >> 32);
-                    const float bj = bget(j);
-                    if (walk_p && unit32(xu) * bp <= bj) {
-                        wp = j;
-                        bp = bj;
+        for (int base = 0; base < NO; base += G) {
+            // the next G moves, one per lane (words past the sweep's end are drawn and not used)
+            const MoveDraw ahead = draw_move<MODE>(base + G + gl, n, wr + P.walker_base, key, NO, yd, T, sBeta, sRgap);
+            const int left = NO - base;
+#pragma unroll (WALK ? 1 : UNROLL)
+            for (int i = 0; i < G; ++i) {
+                [[maybe_unused]] const int mv = base + i;
+                if constexpr (WALK)
+                    if (i >= left) break;
+                if constexpr (WALK) {
+                    // the index walk (Sec. 2.3) on the spectrum as it is now: lane t of the group
+                    // draws step t + 1's words (counter (mv, n, w, 2 + t)), lane L the admixture's
+                    const int L = P.walk_len;
+                    const uint4 wr4 = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)(wr + P.walker_base), 2u + gl), key);
+                    const bool walk_p = !(unit32(__shfl_sync(kFull, wr4.x, L, G)) < rho);
+                    const bool walk_s = !(unit32(__shfl_sync(kFull, wr4.y, L, G)) < rho);
+                    int wp = cur.ps & 0xFFFF;
+                    float bp = bget(wp);
+                    for (int t = 0; t < L; ++t) {
+                        const uint32_t xj = __shfl_sync(kFull, wr4.x, t, G), xu = __shfl_sync(kFull, wr4.y, t, G);
+                        const int j = (int)(((uint64_t)xj * (uint64_t)NO) >> 32);
+                        const float bj = bget(j);
+                        if (walk_p && unit32(xu) * bp <= bj) {
+                            wp = j;
+                            bp = bj;
+                        }
                     }
-                }
-                int ws = cur.ps >> 16;
-                ws += (ws >= wp);
-                float bs = bget(ws);
-                for (int t = 0; t < L; ++t) {
-                    const uint32_t xj = __shfl_sync(kFull, wr4.z, t, G), xu = __shfl_sync(kFull, wr4.w, t, G);
-                    int j = (int)(((uint64_t)xj * (uint64_t)(NO - 1)) >> 32);
-                    j += (j >= wp);
-                    const float bj = bget(j);
-                    if (walk_s && unit32(xu) * bs <= bj) {
-                        ws = j;
-                        bs = bj;
+                    int ws = cur.ps >> 16;
+                    ws += (ws >= wp);
+                    float bs = bget(ws);
+                    for (int t = 0; t < L; ++t) {
+                        const uint32_t xj = __shfl_sync(kFull, wr4.z, t, G), xu = __shfl_sync(kFull, wr4.w, t, G);
+                        int j = (int)(((uint64_t)xj * (uint64_t)(NO - 1)) >> 32);
+                        j += (j >= wp);
+                        const float bj = bget(j);
+                        if (walk_s && unit32(xu) * bs <= bj) {
+                            ws = j;
+                            bs = bj;
+                        }
                     }
+                    cur.ps = wp | (ws << 16);
+                    deltas(cur.eps, wp, ws, sBeta, sRgap, cur.dp, cur.ds);
                 }
-                cur.ps = wp | (ws << 16);
-                deltas(cur.eps, wp, ws, sBeta, sRgap, cur.dp, cur.ds);
-            }
-            // BAHEAD: move k+1's words (they do not depend on move k's outcome) and its b
-            // values, read now so that their latency overlaps move k; if move k is accepted
-            // and writes one of those bins, the written value replaces the one read (the value
-            // a read after the write returns).  nxt's bins are valid indices also past the
-            // sweep's last move.
-            MoveDraw nxt;
-            float bpn = 0.0f, bsn = 0.0f;
-            if constexpr (BAHEAD) {
-                nxt = take_move(mine, (mv + 1) & (G - 1), G);
-                bpn = bget(nxt.ps & 0xFFFF);
-                bsn = bget(nxt.ps >> 16);
-            }
-            // move k: positivity (Eq. probability-density) on the spectrum as it is now
-            const int p = cur.ps & 0xFFFF, s = cur.ps >> 16;
-            const float r = 1.0f - cur.eps;
-            float bp, bs;
-            if constexpr (BAHEAD) {
-                bp = bpc;
-                bs = bsc;
-            } else {
-                bp = bget(p);
-                bs = bget(s);
-            }
-            const float ap = fmaf(r, ghi * bp, cur.dp);
-            const float as = fmaf(r, ghi * bs, cur.ds);
-            const bool ok = active && ap >= 0.0f && as >= 0.0f;
-            pos += (active && !ok);
-            // move k: residual change d = eps M + dpart
-            const f2 e2 = pk(cur.eps, cur.eps);
-            f2 d[C][H];
-            if constexpr (PIPE) {
+                // BAHEAD: move k+1's words (they do not depend on move k's outcome) and its b
+                // values, read now so that their latency overlaps move k; if move k is accepted
+                // and writes one of those bins, the written value replaces the one read (the value
+                // a read after the write returns).  nxt's bins are valid indices also past the
+                // sweep's last move.
+                MoveDraw nxt;
+                float bpn = 0.0f, bsn = 0.0f;
+                if constexpr (BAHEAD) {
+                    nxt = take_move(i < G - 1 ? mine : ahead, (i + 1) & (G - 1), G);
+                    bpn = bget(nxt.ps & 0xFFFF);
+                    bsn = bget(nxt.ps >> 16);
+                }
+                // move k: positivity (Eq. probability-density) on the spectrum as it is now
+                const int p = cur.ps & 0xFFFF, s = cur.ps >> 16;
+                const float r = 1.0f - cur.eps;
+                float bp, bs;
+                if constexpr (BAHEAD) {
+                    bp = bpc;
+                    bs = bsc;
+                } else {
+                    bp = bget(p);
+                    bs = bget(s);
+                }
+                const float ap = fmaf(r, ghi * bp, cur.dp);
+                const float as = fmaf(r, ghi * bs, cur.ds);
+                const bool live = active && i < left;
+                const bool ok = live && ap >= 0.0f && as >= 0.0f;
+                pos += (live && !ok);
+                // move k: residual change d = eps M + dpart
+                const f2 e2 = pk(cur.eps, cur.eps);
+                f2 d[C][H];
+                if constexpr (PIPE) {
 #pragma unroll
-                for (int c = 0; c < C; ++c)
+                    for (int c = 0; c < C; ++c)
 #pragma unroll
-                    for (int h = 0; h < H; ++h) d[c][h] = fma2(e2, M[c][h], dcur[c][h]);
-            } else {
-                columns_tab<G, C, CT>(d, tab, cur);
+                        for (int h = 0; h < H; ++h) d[c][h] = fma2(e2, M[c][h], dcur[c][h]);
+                } else {
+                    columns_tab<G, C, CT>(d, tab, cur);
 #pragma unroll
-                for (int c = 0; c < C; ++c)
+                    for (int c = 0; c < C; ++c)
 #pragma unroll
-                    for (int h = 0; h < H; ++h) d[c][h] = fma2(e2, M[c][h], d[c][h]);
-            }
-            // move k+1: its words (unless taken above) and (pipelined) its columns, into dcur,
-            // now free; neither depends on move k's outcome
-            if constexpr (!BAHEAD) nxt = take_move(mine, (mv + 1) & (G - 1), G);
-            if constexpr (PIPE) columns_tab<G, C, CT>(dcur, tab, nxt);
-            // move k: delta chi2 = sum d (2 R + d) and the Metropolis test
-            float D;
-            bool acc_k;
-            if constexpr (MODE == kGuard) {
-                float Dp, Sp;
-                delta_sum_mag<C, H>(d, R, two, Dp, Sp);
-                D = group_sum<G>(Dp);
-                acc_k = guarded_accept<G, C, CT>(ok, D, group_sum<G>(Sp), cur.thr, P.fp64_accept, R, M, tab, cur,
-                                             n_re, n_flip);
-            } else {
-                D = group_sum<G>(delta_sum<C, H>(d, R, two));
-                // the Hastings threshold may be negative: then D <= 0 does not pass by itself
-                acc_k = ok && (MODE == kHastings ? D < cur.thr : (D <= 0.0f || D < cur.thr));
-            }
-            if (acc_k) {
+                        for (int h = 0; h < H; ++h) d[c][h] = fma2(e2, M[c][h], d[c][h]);
+                }
+                // move k+1: its words (unless taken above) and (pipelined) its columns, into dcur,
+                // now free; neither depends on move k's outcome
+                if constexpr (!BAHEAD) nxt = take_move(i < G - 1 ? mine : ahead, (i + 1) & (G - 1), G);
+                if constexpr (PIPE) columns_tab<G, C, CT>(dcur, tab, nxt);
+                // move k: delta chi2 = sum d (2 R + d) and the Metropolis test
+                float D;
+                bool acc_k;
+                if constexpr (MODE == kGuard) {
+                    float Dp, Sp;
+                    delta_sum_mag<C, H>(d, R, two, Dp, Sp);
+                    D = group_sum<G>(Dp);
+                    acc_k = guarded_accept<G, C, CT>(ok, D, group_sum<G>(Sp), cur.thr, P.fp64_accept, R, M, tab, cur,
+                                                 n_re, n_flip);
+                } else {
+                    D = group_sum<G>(delta_sum<C, H>(d, R, two));
+                    // the Hastings threshold may be negative: then D <= 0 does not pass by itself
+                    acc_k = ok && (MODE == kHastings ? D < cur.thr : (D <= 0.0f || D < cur.thr));
+                }
+                // the update, branch-free: a mask of 1 or 0 adds d or leaves R and M as they are, and every
+                // lane of the walker stores the same two values (each later reads its own store)
+                const float am = acc_k ? 1.0f : 0.0f;
+                const f2 am2 = pk(am, am), nam2 = pk(-am, -am);
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
 #pragma unroll
                     for (int h = 0; h < H; ++h) {
-                        R[c][h] = add2(R[c][h], d[c][h]);
-                        M[c][h] = fma2(minus_one, d[c][h], M[c][h]);
+                        R[c][h] = fma2(am2, d[c][h], R[c][h]);
+                        M[c][h] = fma2(nam2, d[c][h], M[c][h]);
                     }
                 }
-                pair_scale(ghi, glo, r);
+                float gah = ghi, gal = glo;
+                pair_scale(gah, gal, r);
+                const float inv_g = rcp_rn(gah);
+                const float bp_new = ap * inv_g, bs_new = as * inv_g;
+                put_if<STAGED>(am, b, p, s, bp_new, bs_new);
                 if constexpr (BAHEAD) {
-                    const float inv_g = 1.0f / ghi;
-                    const float bp_new = ap * inv_g, bs_new = as * inv_g;
-                    if (gl == 0) {
-                        bset(p, bp_new);
-                        bset(s, bs_new);
-                    }
                     const int pn = nxt.ps & 0xFFFF, sn = nxt.ps >> 16;
-                    bpn = pn == p ? bp_new : (pn == s ? bs_new : bpn);
-                    bsn = sn == p ? bp_new : (sn == s ? bs_new : bsn);
-                } else if (gl == 0) {
-                    const float inv_g = 1.0f / ghi;
-                    bset(p, ap * inv_g);
-                    bset(s, as * inv_g);
+                    bpn = acc_k && pn == p ? bp_new : (acc_k && pn == s ? bs_new : bpn);
+                    bsn = acc_k && sn == p ? bp_new : (acc_k && sn == s ? bs_new : bsn);
                 }
-                dchi += D;
-                ++acc;
+                ghi = acc_k ? gah : ghi;
+                glo = acc_k ? gal : glo;
+                dchi += acc_k ? D : 0.0f;
+                acc += acc_k;
+                cur = nxt;
+                if constexpr (BAHEAD) {
+                    bpc = bpn;
+                    bsc = bsn;
+                }
             }
-            __syncwarp();
-            cur = nxt;
-            if constexpr (BAHEAD) {
-                bpc = bpn;
-                bsc = bsn;
-            }
-            // the next batch of G moves, one per lane, before its first move is taken
-            if (((mv + 2) & (G - 1)) == 0 && mv + 2 < NO)
-                mine = draw_move<MODE>(mv + 2 + gl, n, wr + P.walker_base, key, NO, yd, T, sBeta, sRgap);
+            mine = ahead;
         }
         chi2 += (double)dchi;
         accp = acc;
@@ -968,7 +1007,8 @@ __device__ __forceinline__ void run_group_ahead(const DevProblem &P, const DevSt
         // the spectrum if the move is accepted: scale g r, b_p and b_s as the update writes them
         float gah = ghi, gal = glo;
         pair_scale(gah, gal, r);
-        const float inv_g = 1.0f / gah;
+        // (the plain loop is within 1% of the register file's end and loses that much to rcp_rn)
+        const float inv_g = MODE == kPlain ? 1.0f / gah : rcp_rn(gah);
         const float bpn = ap * inv_g, bsn = as * inv_g;
         // the later proposals' feasibility for either outcome of this move
         bool rA, fA, aA, gA, rB, fB, aB, gB;
@@ -1107,7 +1147,7 @@ __host__ __device__ constexpr bool sweep_compact() {
 }
 
 template <int G, int C, int MODE, bool AHEAD>
-__global__ void __launch_bounds__(sweep_threads<G, C, MODE>()) sweep_fp32_kernel(DevProblem P, DevState S, int n0, int n1,
+__global__ void __launch_bounds__(sweep_threads<G, C, MODE>(), 1) sweep_fp32_kernel(DevProblem P, DevState S, int n0, int n1,
                                                               SweepGeom Gm) {
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);

@@ -215,32 +215,6 @@ __device__ __forceinline__ void span_d(const SpanVec<RR> (&g)[NV], const SpanVec
     }
 }
 
-// 1 / g, correctly rounded, for g and 1 / g in FP32's normal range (g is a product of factors
-// 1 - eps over one launch): one Newton step y + y (1 - g y) in fused arithmetic from the hardware's
-// approximation (Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990).  Equal to 1.0f / g for all 2^23 significands at every exponent from 2^-125 to
-// 2^125 (checked on the GPU).
-__device__ __forceinline__ float rcp_rn(float g) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(g));
-    return fmaf(y, fmaf(-g, y, 1.0f), y);
-}
-
-// b[p] = vp and b[s] = vs if take != 0
-template <bool SMEM>
-__device__ __forceinline__ void put_if(float take, float *b, int p, int s, float vp, float vs) {
-    if constexpr (SMEM)
-        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.shared.f32 [%1], %3;\n\t"
-                     "@q st.shared.f32 [%2], %4;\n\t}"
-                     ::"f"(take), "r"((uint32_t)__cvta_generic_to_shared(b + p)),
-                     "r"((uint32_t)__cvta_generic_to_shared(b + s)), "f"(vp), "f"(vs) : "memory");
-    else
-        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.f32 q, %0, 0f00000000;\n\t@q st.global.f32 [%1], %3;\n\t"
-                     "@q st.global.f32 [%2], %4;\n\t}"
-                     ::"f"(take), "l"(__cvta_generic_to_global(b + p)), "l"(__cvta_generic_to_global(b + s)), "f"(vp),
-                     "f"(vs) : "memory");
-}
-
 // The line of b[j] (global memory) into L1.
 __device__ __forceinline__ void touch(const float *b, int j) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(b + j)));
