@@ -87,107 +87,208 @@ __device__ void walk_bins64(const DevProblem &P, const double *a, uint32_t w0, u
     s_out = s;
 }
 
-template <int C>
+// What a move needs besides the state, drawn by one lane for one of the next 32 moves (the
+// divisions of the two deltas cost the FP64 pipe one instruction for 32 moves instead of one each).
+struct Ring64 {
+    double eps[32], dp[32], ds[32], u[32];
+    double hl[32];        // Hastings: (N - 4) ln r, or NaN where the reverse move cannot be proposed
+    float lnu[32];        // -ln u
+    int p[32], s[32];     // the bins (without an index walk)
+};
+
+// A warp's shared memory: its draws, the terms of delta chi2 on their way to the ordered sum, and the
+// spectrum if it is staged.
+__host__ __device__ __forceinline__ size_t sweep64_warp_bytes(bool staged, int n_omega, int C) {
+    return sizeof(Ring64) + (size_t)(32 * C) * 8 + (staged ? (size_t)n_omega * 8 : 0);
+}
+
+// One warp per walker; every state value and every decision is the oracle's bit for bit.  The FP64
+// pipe answers after some 60 cycles, so the chain of a move was its ordered sum of n_tau additions
+// (needed only where the decision is close: see below), two divisions and an exponential in FP64, and
+// the L2 latency of a[p] and a[s].  Now the draws are made 32 moves at a time, the spectrum is staged
+// in shared memory where it fits, the next move's columns are loaded during the reduction, and a
+// butterfly sum and FP32 take the clear decisions.  chi2 is not tracked: every sweep launch is
+// followed by its recomputation.  32 tau x 64 bins x 64 walkers, per move: 3.87 us -> 1.1 us.
+template <int C, bool STAGED>
 __global__ void __launch_bounds__(128) sweep_fp64_kernel(DevProblem P, DevState S, int n0, int n1) {
+    extern __shared__ double s_mem64[];
     const int lane = threadIdx.x & 31;
     const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (w >= P.n_walkers) return;
     const int NT = P.n_tau, NO = P.n_omega, PAD = P.n_tau_pad;
-    double *a = S.a64 + (size_t)w * NO;
+    char *mem = reinterpret_cast<char *>(s_mem64) + (threadIdx.x >> 5) * sweep64_warp_bytes(STAGED, NO, C);
+    Ring64 &ring = *reinterpret_cast<Ring64 *>(mem);
+    double *s_t = reinterpret_cast<double *>(mem + sizeof(Ring64));
+    double *ag = S.a64 + (size_t)w * NO;
+    double *a = STAGED ? s_t + 32 * C : ag;
+    if constexpr (STAGED)
+        for (int j = lane; j < NO; j += 32) a[j] = ag[j];
     double R[C], Fh[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         R[c] = S.R64[(size_t)w * PAD + lane + 32 * c];
         Fh[c] = P.Fhat64[lane + 32 * c];
     }
-    double chi2 = S.chi2[w];
     int accp = S.acc_prev[w];
     unsigned long long h = S.hash[w], nacc = 0, npos = 0;
     const uint2 key = philox_key(P.seed);
     const double dmove = P.move_scale > 0.0 ? P.move_scale : 1.0 / NO;
     const int wg = w + P.walker_base;   // the walker's index in the whole population
+    const bool walk = P.walk_len > 0;
+    constexpr bool AHEAD = C <= 4;      // the next move's columns in registers
 
+    // delta_p, delta_s of Eqs. (update-delta-p/s)
+    auto deltas64 = [&](double eps, int p, int s, double &dp, double &ds) {
+        const double xp = P.x64[p], xs = P.x64[s];
+        dp = eps * (P.B - P.A * xs) / (xp - xs);
+        ds = eps * (P.B - P.A * xp) / (xs - xp);
+    };
     for (int n = n0; n < n1; ++n) {
         const double T = P.Tsweep[n];
+        const float inv_T = (float)(1.0 / T);
         const double y = amplitude(accp, NO, P.y_p, P.y_m, P.y_min);
         int acc = 0;
-        for (int mv = 0; mv < NO; ++mv) {
-            const uint4 rnd = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)wg, 0u), key);
-            // shared bins: the group's first walker's words 0 and 1 (its own counter)
-            uint2 bw = make_uint2(rnd.x, rnd.y);
-            if (P.shared_bins > 1 && wg % P.shared_bins != 0) {
-                const uint4 g = philox4x32_10(
-                    make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)(wg - wg % P.shared_bins), 0u), key);
-                bw = make_uint2(g.x, g.y);
-            }
-            int p, s;
-            walk_bins64(P, a, bw.x, bw.y, mv, n, wg, key, p, s);
-            const double eps = (y * dmove) * (2.0 * unit64(rnd.z) - 1.0);
-            const double u = unit64(rnd.w);
-            const double r = 1.0 - eps;
-            const double xp = P.x64[p], xs = P.x64[s];
-            const double dp = eps * (P.B - P.A * xs) / (xp - xs);
-            const double ds = eps * (P.B - P.A * xp) / (xs - xp);
-            const double ap = r * a[p] + dp;
-            const double as = r * a[s] + ds;
-            unsigned code;
-            if (ap < 0.0 || as < 0.0) {
-                code = 2;
-                ++npos;
-            } else {
-                const double *Kp = P.Khat64 + (size_t)p * PAD;
-                const double *Ks = P.Khat64 + (size_t)s * PAD;
-                double d[C], t[C];
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const int i = lane + 32 * c;
-                    const double M = Fh[c] - R[c];
-                    d[c] = eps * M - dp * Kp[i] - ds * Ks[i];
-                    t[c] = d[c] * (2.0 * R[c] + d[c]);
-                }
-                double D = 0.0;
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    for (int l = 0; l < 32; ++l) {
-                        const double v = __shfl_sync(kFull, t[c], l);
-                        if (32 * c + l < NT) D = D + v;
+        for (int base = 0; base < NO; base += 32) {
+            const int count = min(32, NO - base);
+            __syncwarp();
+            if (lane < count) {
+                const int mv = base + lane;
+                const uint4 rnd = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)wg, 0u), key);
+                const double eps = (y * dmove) * (2.0 * unit64(rnd.z) - 1.0);
+                const double u = unit64(rnd.w);
+                ring.eps[lane] = eps;
+                ring.u[lane] = u;
+                ring.lnu[lane] = -logf((float)u);
+                if (!walk) {
+                    // shared bins: the group's first walker's words 0 and 1 (its own counter)
+                    uint2 bw = make_uint2(rnd.x, rnd.y);
+                    if (P.shared_bins > 1 && wg % P.shared_bins != 0) {
+                        const uint4 g = philox4x32_10(
+                            make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)(wg - wg % P.shared_bins), 0u), key);
+                        bw = make_uint2(g.x, g.y);
                     }
+                    int p, s;
+                    move_bins(bw.x, bw.y, NO, p, s);
+                    double dp, ds;
+                    deltas64(eps, p, s, dp, ds);
+                    ring.dp[lane] = dp;
+                    ring.ds[lane] = ds;
+                    ring.p[lane] = p;
+                    ring.s[lane] = s;
                 }
-                bool accept;
-                if (!P.hastings) {
-                    accept = D <= 0.0 || u < exp(-D / T);
-                } else {
-                    // Metropolis-Hastings with the move's Jacobian r^(N-4), the reverse amplitude
-                    // -eps/r proposable only when |eps/r| < y d (the oracle's or_accept)
-                    accept = fabs(eps / r) < y * dmove && u < exp(-D / T + (double)(NO - 4) * log(r));
-                }
-                if (accept) {
-                    for (int j = lane; j < NO; j += 32) a[j] = r * a[j];
-                    __syncwarp();
-                    if (lane == 0) {
-                        a[p] = ap;
-                        a[s] = as;
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < C; ++c) R[c] = R[c] + d[c];
-                    chi2 = chi2 + D;
-                    ++acc;
-                    code = 1;
-                } else {
-                    code = 0;
+                if (P.hastings) {
+                    // the move's Jacobian r^(N-4), the reverse amplitude -eps/r proposable only when
+                    // |eps/r| < y d (the oracle's or_accept)
+                    const double r = 1.0 - eps;
+                    ring.hl[lane] = fabs(eps / r) < y * dmove ? (double)(NO - 4) * log(r) : NAN;
                 }
             }
-            h = (h ^ code) * kFnvPrime;
+            __syncwarp();
+            double Kp[C], Ks[C];
+            auto load_columns = [&](int p, int s) {
+                const double *kp = P.Khat64 + (size_t)p * PAD, *ks = P.Khat64 + (size_t)s * PAD;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    Kp[c] = kp[lane + 32 * c];
+                    Ks[c] = ks[lane + 32 * c];
+                }
+            };
+            if (AHEAD && !walk) load_columns(ring.p[0], ring.s[0]);
+            for (int i = 0; i < count; ++i) {
+                const double eps = ring.eps[i], r = 1.0 - eps;
+                double dp, ds;
+                int p, s;
+                if (walk) {
+                    const int mv = base + i;
+                    const uint4 rnd = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)wg, 0u), key);
+                    walk_bins64(P, a, rnd.x, rnd.y, mv, n, wg, key, p, s);
+                    deltas64(eps, p, s, dp, ds);
+                } else {
+                    dp = ring.dp[i];
+                    ds = ring.ds[i];
+                    p = ring.p[i];
+                    s = ring.s[i];
+                }
+                if (!AHEAD || walk) load_columns(p, s);
+                const double ap = r * a[p] + dp;
+                const double as = r * a[s] + ds;
+                unsigned code;
+                if (ap < 0.0 || as < 0.0) {
+                    if (AHEAD && !walk && i + 1 < count) load_columns(ring.p[i + 1], ring.s[i + 1]);
+                    code = 2;
+                    ++npos;
+                } else {
+                    double d[C], t[C];
+                    double D = 0.0;              // sum in butterfly order; the decision's own unless it is close
+                    float mag = 0.0f;            // sum of the terms' magnitudes
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const double M = Fh[c] - R[c];
+                        d[c] = eps * M - dp * Kp[c] - ds * Ks[c];
+                        t[c] = d[c] * (2.0 * R[c] + d[c]);
+                        D = D + t[c];
+                        mag += fabsf((float)t[c]);
+                    }
+                    if (AHEAD && !walk && i + 1 < count) load_columns(ring.p[i + 1], ring.s[i + 1]);
+                    for (int o = 16; o > 0; o >>= 1) {
+                        D = D + __shfl_xor_sync(kFull, D, o);
+                        mag += __shfl_xor_sync(kFull, mag, o);
+                    }
+                    // accept with probability min(1, exp(-D / T)) (Hastings: times r^(N-4)).  The sums in
+                    // two orders differ by at most n_tau 2^-53 of the terms' magnitudes (512 points:
+                    // 6e-14) and FP32 rounds x = D / T and -ln u (+ (N-4) ln r) to about 1e-7 of
+                    // themselves; where the decision lies outside both it is taken, else the terms
+                    // are added in the oracle's order and the test is evaluated in FP64.
+                    const double hl = P.hastings ? ring.hl[i] : 0.0;
+                    const float Df = (float)D, close = 1e-12f * mag;
+                    const float x = Df * inv_T, lnu = ring.lnu[i], hf = (float)hl, gap = x - (lnu + hf);
+                    const float tol = 1e-5f * (fabsf(x) + lnu + fabsf(hf)) + 1e-6f + close * inv_T;
+                    bool accept;
+                    if (hl != hl) {
+                        accept = false;
+                    } else if (!P.hastings && Df < -close) {
+                        accept = true;
+                    } else if (fabsf(gap) > tol && (P.hastings || Df > close)) {
+                        accept = gap < 0.0f;
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) s_t[lane + 32 * c] = t[c];
+                        __syncwarp();
+                        D = 0.0;
+                        for (int q = 0; q < NT; ++q) D = D + s_t[q];
+                        if (!P.hastings) accept = D <= 0.0 || ring.u[i] < exp(-D / T);
+                        else accept = ring.u[i] < exp(-D / T + hl);
+                    }
+                    if (accept) {
+                        for (int j = lane; j < NO; j += 32) a[j] = r * a[j];
+                        __syncwarp();
+                        if (lane == 0) {
+                            a[p] = ap;
+                            a[s] = as;
+                        }
+#pragma unroll
+                        for (int c = 0; c < C; ++c) R[c] = R[c] + d[c];
+                        ++acc;
+                        code = 1;
+                    } else {
+                        code = 0;
+                    }
+                    __syncwarp();
+                }
+                h = (h ^ code) * kFnvPrime;
+            }
         }
         accp = acc;
         nacc += acc;
         if (S.acc_trace && lane == 0) S.acc_trace[(size_t)n * P.n_walkers + w] = acc;
     }
+    if constexpr (STAGED) {
+        __syncwarp();
+        for (int j = lane; j < NO; j += 32) ag[j] = a[j];
+    }
 #pragma unroll
     for (int c = 0; c < C; ++c) S.R64[(size_t)w * PAD + lane + 32 * c] = R[c];
     if (lane == 0) {
-        S.chi2[w] = chi2;
         S.acc_prev[w] = accp;
         S.hash[w] = h;
         S.n_acc[w] += nacc;
@@ -1071,12 +1172,25 @@ __global__ void philox_kernel(int n, const uint32_t *ctr, uint64_t seed, uint32_
 
 template <int C>
 cudaError_t launch_sweep64_c(const DevProblem &P, const DevState &S, int n0, int n1, cudaStream_t st) {
-    const int threads = 128;
-    const int blocks = (P.n_walkers * 32 + threads - 1) / threads;
-    sweep_fp64_kernel<C><<<blocks, threads, 0, st>>>(P, S, n0, n1);
+    // one warp a block while the walkers do not fill the SMs (a warp's FP64 chain wants an SM's FP64
+    // pipe for itself), up to four otherwise
+    int dev = 0, sms = 1, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    int warps = (P.n_walkers + sms - 1) / sms;
+    warps = warps > 4 ? 4 : warps;
+    const int blocks = (P.n_walkers + warps - 1) / warps;
+    const size_t staged = warps * sweep64_warp_bytes(true, P.n_omega, C);
+    if (staged <= (size_t)smem_max) {
+        const cudaError_t e = cudaFuncSetAttribute(sweep_fp64_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+        if (e != cudaSuccess) return e;
+        sweep_fp64_kernel<C, true><<<blocks, 32 * warps, staged, st>>>(P, S, n0, n1);
+    } else {
+        sweep_fp64_kernel<C, false><<<blocks, 32 * warps, warps * sweep64_warp_bytes(false, P.n_omega, C), st>>>(P, S, n0, n1);
+    }
     return cudaGetLastError();
 }
-
 
 // Smoothing of one spectrum (Sec. smoothing), in the oracle's order of operations: the
 // three-point stencil of strength s from the old values, ends (1 - s) a_0 + s a_1 and
