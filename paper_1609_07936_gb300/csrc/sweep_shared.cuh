@@ -98,6 +98,11 @@ __device__ __forceinline__ void run_shared(const DevProblem &P, const DevState &
     constexpr int Q = W / 2;           // walker pairs
     constexpr int LW = W == 8 ? 3 : (W == 4 ? 2 : 1);  // log2 W
     constexpr int MPD = 32 / W;        // moves one draw round covers
+    // Four moves a basic block, without a branch for the accepted walkers or the division, where the
+    // registers allow it: 200 tau x 1000 bins x 4096 walkers, 20 sweeps, groups of 8 10.07 -> 7.66 ms,
+    // of 4 8.37 -> 8.07 (50 hot sweeps 22.3 -> 20.1), 1500 walkers 6.90 -> 5.90.  Groups of 2 (10.5 ->
+    // 11.4), the Hastings test (8.6 -> 9.0) and more than 8 chunks (22.5 -> 24.2) lose by it.
+    constexpr bool STRAIGHT = W >= 4 && C <= 8 && MODE == kPlain;
     const int NO = P.n_omega, PAD = P.n_tau_pad, NH = (NO + 31) >> 5;
     const float *sQhi = sm;
     const float *sQlo = sQhi + (size_t)NH * PAD;
@@ -155,7 +160,7 @@ __device__ __forceinline__ void run_shared(const DevProblem &P, const DevState &
         // next round
         SharedDraw cur = shared_draw<MODE>(q, n, w + P.walker_base, key, NO, yd, T);
         SharedDraw nxt = cur;
-        if (MPD < NO) nxt = shared_draw<MODE>(MPD + q, n, w + P.walker_base, key, NO, yd, T);
+        nxt = shared_draw<MODE>(MPD + q, n, w + P.walker_base, key, NO, yd, T);
         f2 Ga[C], Gb[C];
         float cpa, csa, gga, cpb = 0.0f, csb = 0.0f, ggb = 0.0f;
         const int ps0 = __shfl_sync(kFull, cur.ps, 0);
@@ -166,9 +171,11 @@ __device__ __forceinline__ void run_shared(const DevProblem &P, const DevState &
         auto move = [&](const int mv, f2 (&G)[C], f2 (&Gn)[C], float &cp, float &cs, float &gg, float &cpn,
                         float &csn, float &ggn) {
             const int m = mv & (MPD - 1);
-            if (m == 0 && mv > 0) {
-                cur = nxt;
-                if (mv + MPD < NO) nxt = shared_draw<MODE>(mv + MPD + q, n, w + P.walker_base, key, NO, yd, T);
+            if constexpr (!STRAIGHT) {
+                if (m == 0 && mv > 0) {
+                    cur = nxt;
+                    if (mv + MPD < NO) nxt = shared_draw<MODE>(mv + MPD + q, n, w + P.walker_base, key, NO, yd, T);
+                }
             }
             // this move: the shared bins, every walker's amplitude, this lane's walker's threshold
             const int ps = __shfl_sync(kFull, cur.ps, W * m);
@@ -178,14 +185,14 @@ __device__ __forceinline__ void run_shared(const DevProblem &P, const DevState &
                 e2[j] = pk(__shfl_sync(kFull, cur.eps, 2 * j + W * m), __shfl_sync(kFull, cur.eps, 2 * j + 1 + W * m));
             const float eps = __shfl_sync(kFull, cur.eps, v + W * m);
             const float thr = __shfl_sync(kFull, cur.thr, v + W * m);
-            // the next move's bins (after the sweep's last move: this move's again, unused) and
+            // the next move's bins (past the sweep's end: bins that no live move uses) and
             // this lane's walker's b values there, read now so that their latency overlaps this
             // move (measured at 512 tau x 2048 bins x 16384 walkers, groups of 4, spectra in
             // global memory: +10%); if this move is accepted and writes one of those bins, the
             // written value replaces the one read (the value a read after the write returns)
             const int nps_cur = __shfl_sync(kFull, cur.ps, (W * (m + 1)) & 31);
             const int nps_nxt = __shfl_sync(kFull, nxt.ps, 0);
-            const int nps = mv + 1 >= NO ? ps : (m + 1 < MPD ? nps_cur : nps_nxt);
+            const int nps = !STRAIGHT && mv + 1 >= NO ? ps : (m + 1 < MPD ? nps_cur : nps_nxt);
             float bpn = bget(nps & 0xFFFF), bsn = bget(nps >> 16);
             // every walker's G.R
             f2 acc2[Q];
@@ -227,44 +234,87 @@ __device__ __forceinline__ void run_shared(const DevProblem &P, const DevState &
             const float r = 1.0f - eps;
             const float ap = fmaf(r, ghi * bpc, eps * cs);
             const float as = fmaf(r, ghi * bsc, -(eps * cp));
-            const bool ok = active && ap >= 0.0f && as >= 0.0f;
-            pos += (active && !ok);
+            const bool live = active && (!STRAIGHT || mv < NO);
+            const bool ok = live && ap >= 0.0f && as >= 0.0f;
+            pos += (live && !ok);
             const bool accepted = ok && (MODE == kHastings ? D < thr : (D <= 0.0f || D < thr));
             const unsigned amask = __ballot_sync(kFull, accepted) & ((1u << W) - 1u);
-            if (accepted) {
-                pair_scale(ghi, glo, r);
-                const float inv_g = 1.0f / ghi;
+            if constexpr (STRAIGHT) {
+                // the update without a branch: selects, stores under a predicate (every lane of a walker
+                // stores the same values and later reads its own), and masked residual updates
+                float gah = ghi, gal = glo;
+                pair_scale(gah, gal, r);
+                const float inv_g = rcp_rn(gah);
                 const float bp_new = ap * inv_g, bs_new = as * inv_g;
-                if (q == 0) {
-                    bset(p, bp_new);
-                    bset(sb, bs_new);
-                }
+                put_if<STAGED>(accepted ? 1.0f : 0.0f, b, p, sb, bp_new, bs_new);
                 const int pn = nps & 0xFFFF, sn = nps >> 16;
-                bpn = pn == p ? bp_new : (pn == sb ? bs_new : bpn);
-                bsn = sn == p ? bp_new : (sn == sb ? bs_new : bsn);
-                dchi += D;
-                chi2f += D;
-                ++acc;
-            }
-            // accepted walkers: R <- R + eps (G - R)
+                bpn = accepted && pn == p ? bp_new : (accepted && pn == sb ? bs_new : bpn);
+                bsn = accepted && sn == p ? bp_new : (accepted && sn == sb ? bs_new : bsn);
+                ghi = accepted ? gah : ghi;
+                glo = accepted ? gal : glo;
+                dchi += accepted ? D : 0.0f;
+                chi2f += accepted ? D : 0.0f;
+                acc += accepted;
+                // accepted walkers: R <- R + eps (G - R)
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                if (amask & (3u << (2 * j))) {
+                for (int j = 0; j < Q; ++j) {
                     const float2 e = up(e2[j]);
                     const f2 ea = pk((amask >> (2 * j)) & 1u ? e.x : 0.0f, (amask >> (2 * j + 1)) & 1u ? e.y : 0.0f);
 #pragma unroll
                     for (int c = 0; c < C; ++c) R[c][j] = fma2(ea, fma2(minus_one, R[c][j], G[c]), R[c][j]);
+                }
+            } else {
+                if (accepted) {
+                    pair_scale(ghi, glo, r);
+                    const float inv_g = 1.0f / ghi;
+                    const float bp_new = ap * inv_g, bs_new = as * inv_g;
+                    if (q == 0) {
+                        bset(p, bp_new);
+                        bset(sb, bs_new);
+                    }
+                    const int pn = nps & 0xFFFF, sn = nps >> 16;
+                    bpn = pn == p ? bp_new : (pn == sb ? bs_new : bpn);
+                    bsn = sn == p ? bp_new : (sn == sb ? bs_new : bsn);
+                    dchi += D;
+                    chi2f += D;
+                    ++acc;
+                }
+                // accepted walkers: R <- R + eps (G - R)
+#pragma unroll
+                for (int j = 0; j < Q; ++j) {
+                    if (amask & (3u << (2 * j))) {
+                        const float2 e = up(e2[j]);
+                        const f2 ea = pk((amask >> (2 * j)) & 1u ? e.x : 0.0f, (amask >> (2 * j + 1)) & 1u ? e.y : 0.0f);
+#pragma unroll
+                        for (int c = 0; c < C; ++c) R[c][j] = fma2(ea, fma2(minus_one, R[c][j], G[c]), R[c][j]);
+                    }
                 }
             }
             __syncwarp();
             bpc = bpn;
             bsc = bsn;
         };
-        for (int mv = 0; mv + 1 < NO; mv += 2) {
-            move(mv, Ga, Gb, cpa, csa, gga, cpb, csb, ggb);
-            move(mv + 1, Gb, Ga, cpb, csb, ggb, cpa, csa, gga);
+        if constexpr (STRAIGHT) {
+            // rounds of MPD moves without a branch between them (moves past the sweep's end are not
+            // live), four moves a basic block
+            for (int mv0 = 0; mv0 < NO; mv0 += MPD) {
+                if (mv0 > 0) {
+                    cur = nxt;
+                    nxt = shared_draw<MODE>(mv0 + MPD + q, n, w + P.walker_base, key, NO, yd, T);
+                }
+#pragma unroll 2
+                for (int m = 0; m < MPD; m += 2) {
+                    move(mv0 + m, Ga, Gb, cpa, csa, gga, cpb, csb, ggb);
+                    move(mv0 + m + 1, Gb, Ga, cpb, csb, ggb, cpa, csa, gga);
+                }
+            }
+        } else {
+            for (int mv = 0; mv + 1 < NO; mv += 2) {
+                move(mv, Ga, Gb, cpa, csa, gga, cpb, csb, ggb);
+                move(mv + 1, Gb, Ga, cpb, csb, ggb, cpa, csa, gga);
+            }
+            if (NO & 1) move(NO - 1, Ga, Gb, cpa, csa, gga, cpb, csb, ggb);
         }
-        if (NO & 1) move(NO - 1, Ga, Gb, cpa, csa, gga, cpb, csb, ggb);
         chi2 += (double)dchi;
         accp = acc;
         nacc += acc;
