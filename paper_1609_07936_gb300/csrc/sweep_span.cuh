@@ -215,11 +215,6 @@ __device__ __forceinline__ void span_d(const SpanVec<RR> (&g)[NV], const SpanVec
     }
 }
 
-// The line of b[j] (global memory) into L1.
-__device__ __forceinline__ void touch(const float *b, int j) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(b + j)));
-}
-
 // Lane's draw of move mv of walker wr.  The Metropolis test is D < threshold: D <= 0 passes, so a
 // plain threshold is at least the smallest positive float (the Hastings threshold may be negative).
 // Past the sweep's end, and for walkers that do not exist, a null move: eps = 1 makes its
@@ -280,9 +275,11 @@ __device__ __forceinline__ void span_write_back(const DevProblem &P, const DevSt
 // Sweeps [n0, n1) for the 32 / G walkers of group grp of one problem on one warp.
 //   tab    the column table (shared memory if TS, else global memory), rows of RR floats
 //   sBeta, sRgap  beta and the reciprocal gaps (shared memory)
-//   b      STAGED: the spectra of walkers walker_lo.. in shared memory; else in global memory,
-//          where a move's b_p, b_s are read one move ahead (and patched if the move before it
-//          writes one of those bins), from lines fetched into L1 a move earlier still
+//   b      STAGED: the spectra of walkers walker_lo.. in shared memory.  Else in global memory,
+//          where a read takes longer than several moves; each lane reads b_p, b_s of the move it
+//          drew a batch ahead and keeps them, replaces them when a move before it writes one of
+//          those bins (until the batch turns over the replacement waits apart, so that nothing
+//          waits for the read), and hands them over by shuffle
 // Every lane of a walker writes an accepted move's two amplitudes (the same values), so each
 // lane later reads its own write and the loop needs no barrier.
 template <int RR, int G, bool TS, bool STAGED, int MODE>
@@ -293,7 +290,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
     static_assert(MODE != kWalk || G == 8, "the walk's words are drawn by 8 lanes");
     constexpr int WPW = 32 / G, NV = 8 / G;
     constexpr bool WALK = MODE == kWalk;
-    constexpr bool BAHEAD = !STAGED && !WALK;
+    constexpr bool OWN = !STAGED && !WALK;      // b_p, b_s held by the lane that drew the move (above)
     using V = SpanVec<RR>;
     const int NO = P.n_omega;
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), sub = lane / G;
@@ -323,19 +320,29 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
         const float yd = (float)(amplitude(accp, NO, P.y_p, P.y_m, P.y_min) * dmove);
         int acc = 0, pos = 0;
         __syncwarp();
-        span_put(ring, 0, span_draw<MODE>(P, gl, n, wr, active, key, yd, T, sBeta, sRgap));
+        const MoveDraw first = span_draw<MODE>(P, gl, n, wr, active, key, yd, T, sBeta, sRgap);
+        span_put(ring, 0, first);
         __syncwarp();
         SpanMove cur = span_get<G>(ring, 0, 0), nxt = span_get<G>(ring, 0, 1);
         V g[NV];
         if constexpr (!WALK) span_g<RR, NV, TS>(tab, vl, F, cur, g);
-        float bpc = 0.0f, bsc = 0.0f;          // BAHEAD: b at the current move's bins
-        if constexpr (BAHEAD) {
-            bpc = b[cur.ps & 0xFFFF];
-            bsc = b[cur.ps >> 16];
+        // OWN: this lane's move of the batch: its bins and b there
+        int own_p = first.ps & 0xFFFF, own_s = first.ps >> 16;
+        float own_bp = 0.0f, own_bs = 0.0f;
+        if constexpr (OWN) {
+            own_bp = b[own_p];
+            own_bs = b[own_s];
         }
         int batch = 0;
         for (int base = 0; base < NO; base += G, batch ^= 1) {
             const MoveDraw mine = span_draw<MODE>(P, base + G + gl, n, wr, active, key, yd, T, sBeta, sRgap);
+            // OWN: b at the next batch's move, read now, and what this batch's moves write there meanwhile
+            const int next_p = mine.ps & 0xFFFF, next_s = mine.ps >> 16;
+            float next_bp = 0.0f, next_bs = 0.0f, new_bp = __int_as_float(-1), new_bs = __int_as_float(-1);
+            if constexpr (OWN) {
+                next_bp = b[next_p];
+                next_bs = b[next_s];
+            }
 #pragma unroll
             for (int i = 0; i < G; ++i) {
                 if (i == (G > 4 ? G - 3 : 1)) {
@@ -390,22 +397,16 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 float D = span_part<RR>(d[0], R[0], C[0], two);
                 if constexpr (NV == 2) D += span_part<RR>(d[1], R[1], C[1], two);
                 const int p = cur.ps & 0xFFFF, s = cur.ps >> 16;
-                float bp, bs, bpn = 0.0f, bsn = 0.0f;
-                if constexpr (BAHEAD) {
-                    bp = bpc;
-                    bs = bsc;
-                    bpn = b[nxt.ps & 0xFFFF];
-                    bsn = b[nxt.ps >> 16];
+                float bp, bs;
+                if constexpr (OWN) {
+                    bp = __shfl_sync(kFull, own_bp, i, G);
+                    bs = __shfl_sync(kFull, own_bs, i, G);
                 } else {
                     bp = b[p];
                     bs = b[s];
                 }
                 if constexpr (!WALK) span_g<RR, NV, TS>(tab, vl, F, nxt, g);
                 const SpanMove far = i < G - 2 ? span_get<G>(ring, batch, i + 2) : span_get<G>(ring, batch ^ 1, i + 2 - G);
-                if constexpr (BAHEAD) {
-                    touch(b, far.ps & 0xFFFF);
-                    touch(b, far.ps >> 16);
-                }
                 // positivity (Eq. probability-density) on the spectrum as it is now, and the spectrum
                 // if the move is accepted
                 const float r = 1.0f + cur.me;
@@ -428,13 +429,21 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 ghi = acc_k ? gah : ghi;
                 glo = acc_k ? gal : glo;
                 acc += acc_k;
-                if constexpr (BAHEAD) {
-                    const int pn = nxt.ps & 0xFFFF, sn = nxt.ps >> 16;
-                    bpc = acc_k && pn == p ? ap_b : (acc_k && pn == s ? as_b : bpn);
-                    bsc = acc_k && sn == p ? ap_b : (acc_k && sn == s ? as_b : bsn);
+                if constexpr (OWN) {
+                    const int wp = acc_k ? p : -1, ws = acc_k ? s : -1;
+                    own_bp = own_p == wp ? ap_b : (own_p == ws ? as_b : own_bp);
+                    own_bs = own_s == wp ? ap_b : (own_s == ws ? as_b : own_bs);
+                    new_bp = next_p == wp ? ap_b : (next_p == ws ? as_b : new_bp);
+                    new_bs = next_s == wp ? ap_b : (next_s == ws ? as_b : new_bs);
                 }
                 cur = nxt;
                 nxt = far;
+            }
+            if constexpr (OWN) {
+                own_p = next_p;
+                own_s = next_s;
+                own_bp = __float_as_int(new_bp) == -1 ? next_bp : new_bp;
+                own_bs = __float_as_int(new_bs) == -1 ? next_bs : new_bs;
             }
         }
         accp = acc;
@@ -531,12 +540,11 @@ cudaError_t launch_span_g(const DevProblem &P, const DevState &S, int n0, int n1
 
 // Lanes per walker of a launch (either gives the same trajectories).  8 lanes keep one warp's chain
 // shortest: they run while the spectra are staged and the SM's schedulers have room (20 sweeps, 200
-// x 1000: 1500 walkers 1.98 ms against 2.79 with 4 lanes, 4096: 2.81 against 5.7, which does not
+// x 1000: 1500 walkers 2.01 ms against 2.79 with 4 lanes, 4096: 2.85 against 5.7, which does not
 // stage).  4 lanes need 0.8 of the instructions per walker: they run where the spectra stay in
-// global memory anyway (8192 walkers 6.3 against 7.9 ms, 16384: 9.0 against 15.6; 512 x 2048: 608
-// walkers 11.2 against 14.9, 8192: 13.2 against 19.0), and where the population fills the
-// schedulers and is staged (32 x 64, 200 sweeps: 4096 walkers 1.67 against 1.86 ms; 608: 1.63
-// against 1.36).
+// global memory anyway (8192 walkers 6.1 against 7.9 ms, 16384: 9.0 against 15.6; 512 x 2048: 608
+// walkers 7.9 against 14.9), and where the population fills the schedulers and is staged (32 x 64,
+// 200 sweeps: 4096 walkers 1.70 against 1.86 ms; 608: 1.63 against 1.36).
 template <int RR, int MODE>
 cudaError_t launch_span(const DevProblem &P, const DevState &S, int n0, int n1, cudaStream_t st) {
     int dev = 0, sms = 0, smem_max = 0;
