@@ -27,7 +27,7 @@
 // iteration of four walkers, 290 cycles at two warps on a scheduler, 64% of its issue slots and 67%
 // of the shared-memory data pipe), 16384 walkers 198 -> 45 ms; 512 x 2048 x 16384, 10 sweeps 90 ->
 // 14 ms (spectra in L2); 160 x 1000 x 1500, 100 sweeps 35.5 -> 9.6 ms (203 cycles an iteration,
-// one warp); Hastings 72 -> 15.7 ms; index walk (1500 walkers, 50 sweeps) 47 -> 30 ms.
+// one warp); Hastings 72 -> 15.7 ms; index walk (L = 2, 1500 walkers, 50 sweeps) 47 -> 16 ms.
 //
 // Layout.  G lanes per walker (8 or 4: four or eight walkers a warp).  The RR elements belong to
 // eight virtual lanes, RR / 8 each; delta chi2 is the xor-butterfly sum (4, 2, 1) of the virtual
@@ -253,6 +253,44 @@ __device__ __forceinline__ SpanMove span_get(const SpanRing &ring, int batch, in
     return m;
 }
 
+// The steps of one move's index walk (Sec. 2.3): proposed bins for p and (before skipping p) for s, and
+// the uniforms of their acceptance; a step that is not taken (past P.walk_len, or the whole walk
+// skipped by the uniform admixture) has a NaN, which no proposal passes.
+template <int LM>
+struct SpanSteps {
+    int jp[LM], js[LM];
+    float up[LM], us[LM];
+};
+template <int G, int LM>
+__device__ __forceinline__ SpanSteps<LM> span_steps(const DevProblem &P, int mv, int n, int wr, uint2 key, float rho, int gl) {
+    // lane t of the group draws step t + 1's words (counter (mv, n, w, 2 + t)), lane L the admixture's
+    const int L = P.walk_len, NO = P.n_omega;
+    const uint4 w4 = philox4x32_10(make_uint4((uint32_t)mv, (uint32_t)n, (uint32_t)(wr + P.walker_base), 2u + gl), key);
+    const bool walk_p = !(unit32(__shfl_sync(kFull, w4.x, L, G)) < rho);
+    const bool walk_s = !(unit32(__shfl_sync(kFull, w4.y, L, G)) < rho);
+    const int jp = (int)(((uint64_t)w4.x * (uint64_t)NO) >> 32), js = (int)(((uint64_t)w4.z * (uint64_t)(NO - 1)) >> 32);
+    const float up = walk_p && gl < L ? unit32(w4.y) : NAN, us = walk_s && gl < L ? unit32(w4.w) : NAN;
+    SpanSteps<LM> s;
+#pragma unroll
+    for (int t = 0; t < LM; ++t) {
+        s.jp[t] = __shfl_sync(kFull, jp, t, G);
+        s.js[t] = __shfl_sync(kFull, js, t, G);
+        s.up[t] = __shfl_sync(kFull, up, t, G);
+        s.us[t] = __shfl_sync(kFull, us, t, G);
+    }
+    return s;
+}
+// Move m proposes bins p and s.
+__device__ __forceinline__ void span_walk_to(SpanMove &m, int p, int s, const float *sBeta, const float *sRgap) {
+    float dp, ds;
+    m.ps = p | (s << 16);
+    deltas(-m.me, p, s, sBeta, sRgap, dp, ds);
+    m.mdp = -dp;
+    m.mds = -ds;
+    m.mdp2 = pk(-dp, -dp);
+    m.mds2 = pk(-ds, -ds);
+}
+
 // Folds the common scale into walker w's spectrum b and writes the walker back (lane gl of its G).
 template <int G>
 __device__ __forceinline__ void span_write_back(const DevProblem &P, const DevState &S, int w, int gl, const float *b, float ghi,
@@ -282,7 +320,13 @@ __device__ __forceinline__ void span_write_back(const DevProblem &P, const DevSt
 //          waits for the read), and hands them over by shuffle
 // Every lane of a walker writes an accepted move's two amplitudes (the same values), so each
 // lane later reads its own write and the loop needs no barrier.
-template <int RR, int G, bool TS, bool STAGED, int MODE>
+//
+// LM > 0 (index walk): the walk's steps unrolled to LM >= P.walk_len.  The proposals of a walk do not
+// depend on the state, so the steps' words are drawn and handed out one move ahead, and b at all of
+// them (for s, at the bin and the one after: the proposals skip p) is read at once; what is left on the
+// chain is a comparison a step.  LM = 0: steps in a loop, each with its own reads (the batched sweep).
+// 200 x 1000, 10 sweeps: L = 2, 1500 walkers 6.0 -> 3.2 ms (9.4 over tau), 4096 4.0, L = 7 5.5 (12.1).
+template <int RR, int G, bool TS, bool STAGED, int MODE, int LM = 0>
 __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S, int n0, int n1, int grp,
                                          const float *tab, const float *sBeta, const float *sRgap, SpanRing &ring,
                                          float *b_stage, int walker_lo) {
@@ -333,6 +377,8 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
             own_bp = b[own_p];
             own_bs = b[own_s];
         }
+        SpanSteps<LM == 0 ? 1 : LM> steps;
+        if constexpr (LM > 0) steps = span_steps<G, LM == 0 ? 1 : LM>(P, 0, n, wr, key, rho, gl);
         int batch = 0;
         for (int base = 0; base < NO; base += G, batch ^= 1) {
             const MoveDraw mine = span_draw<MODE>(P, base + G + gl, n, wr, active, key, yd, T, sBeta, sRgap);
@@ -349,7 +395,41 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                     span_put(ring, batch ^ 1, mine);
                     __syncwarp();
                 }
-                if constexpr (WALK) {
+                float walk_bp = 0.0f, walk_bs = 0.0f;
+                if constexpr (WALK && LM > 0) {
+                    const int p0 = cur.ps & 0xFFFF, s0 = cur.ps >> 16;
+                    float bpt[LM], bst[LM], bsu[LM];
+                    float bp = b[p0];
+                    const float b0 = b[s0], b1 = b[s0 + 1];
+#pragma unroll
+                    for (int t = 0; t < LM; ++t) {
+                        bpt[t] = b[steps.jp[t]];
+                        bst[t] = b[steps.js[t]];
+                        bsu[t] = b[steps.js[t] + 1];
+                    }
+                    int wp = p0;
+#pragma unroll
+                    for (int t = 0; t < LM; ++t) {
+                        const bool go = steps.up[t] * bp <= bpt[t];
+                        wp = go ? steps.jp[t] : wp;
+                        bp = go ? bpt[t] : bp;
+                    }
+                    int ws = s0 + (s0 >= wp);
+                    float bs = s0 >= wp ? b1 : b0;
+#pragma unroll
+                    for (int t = 0; t < LM; ++t) {
+                        const bool past = steps.js[t] >= wp;
+                        const float bj = past ? bsu[t] : bst[t];
+                        const bool go = steps.us[t] * bs <= bj;
+                        ws = go ? steps.js[t] + past : ws;
+                        bs = go ? bj : bs;
+                    }
+                    walk_bp = bp;
+                    walk_bs = bs;
+                    span_walk_to(cur, wp, ws, sBeta, sRgap);
+                    span_g<RR, NV, TS>(tab, vl, F, cur, g);
+                    steps = span_steps<G, LM == 0 ? 1 : LM>(P, base + i + 1, n, wr, key, rho, gl);
+                } else if constexpr (WALK) {
                     // the index walk (Sec. 2.3) on the spectrum as it is now: lane t of the group
                     // draws step t + 1's words (counter (mv, n, w, 2 + t)), lane L the admixture's
                     const int mv = base + i;
@@ -381,13 +461,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                             bs = bj;
                         }
                     }
-                    cur.ps = wp | (ws << 16);
-                    float dp, ds;
-                    deltas(-cur.me, wp, ws, sBeta, sRgap, dp, ds);
-                    cur.mdp = -dp;
-                    cur.mds = -ds;
-                    cur.mdp2 = pk(-dp, -dp);
-                    cur.mds2 = pk(-ds, -ds);
+                    span_walk_to(cur, wp, ws, sBeta, sRgap);
                     span_g<RR, NV, TS>(tab, vl, F, cur, g);
                 }
                 // move k: d and its part of delta chi2; then the columns of move k+1 take the place of
@@ -401,6 +475,9 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 if constexpr (OWN) {
                     bp = __shfl_sync(kFull, own_bp, i, G);
                     bs = __shfl_sync(kFull, own_bs, i, G);
+                } else if constexpr (LM > 0) {
+                    bp = walk_bp;
+                    bs = walk_bs;
                 } else {
                     bp = b[p];
                     bs = b[s];
@@ -476,7 +553,7 @@ __device__ __forceinline__ void span_load(const DevProblem &P, float *sBeta, flo
 // floats of the beta and gap vectors, rounded up so that what follows is 16-byte aligned
 __host__ __device__ __forceinline__ int span_vec_floats(int NO) { return (2 * NO + 3) / 4 * 4; }
 
-template <int RR, int G, int MODE>
+template <int RR, int G, int MODE, int LM>
 __global__ void __launch_bounds__(32 * kSpanWarps, 1) sweep_span_kernel(DevProblem P, DevState S, int n0, int n1, SpanGeom Gm) {
     extern __shared__ float4 smem4[];
     constexpr int WPW = 32 / G;
@@ -501,11 +578,11 @@ __global__ void __launch_bounds__(32 * kSpanWarps, 1) sweep_span_kernel(DevProbl
         const int grp = grp_lo + round * Gm.warps + warp;
         if (grp >= grp_hi) break;                         // uniform across the warp
         if (Gm.stage_t && Gm.stage_b)
-            run_span<RR, G, true, true, MODE>(P, S, n0, n1, grp, sTab, sBeta, sRgap, rings[warp], sB, walker_lo);
+            run_span<RR, G, true, true, MODE, LM>(P, S, n0, n1, grp, sTab, sBeta, sRgap, rings[warp], sB, walker_lo);
         else if (Gm.stage_t)
-            run_span<RR, G, true, false, MODE>(P, S, n0, n1, grp, sTab, sBeta, sRgap, rings[warp], nullptr, 0);
+            run_span<RR, G, true, false, MODE, LM>(P, S, n0, n1, grp, sTab, sBeta, sRgap, rings[warp], nullptr, 0);
         else
-            run_span<RR, G, false, false, MODE>(P, S, n0, n1, grp, P.Kspan, sBeta, sRgap, rings[warp], nullptr, 0);
+            run_span<RR, G, false, false, MODE, LM>(P, S, n0, n1, grp, P.Kspan, sBeta, sRgap, rings[warp], nullptr, 0);
     }
 }
 
@@ -528,13 +605,13 @@ SpanGeom span_geom(const DevProblem &P, int sms, int smem_max, size_t *smem) {
     return Gm;
 }
 
-template <int RR, int G, int MODE>
+template <int RR, int G, int MODE, int LM = 0>
 cudaError_t launch_span_g(const DevProblem &P, const DevState &S, int n0, int n1, const SpanGeom &Gm, size_t smem,
                           cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(sweep_span_kernel<RR, G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(sweep_span_kernel<RR, G, MODE, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int n_ctas = (Gm.groups_total + Gm.groups_per_cta - 1) / Gm.groups_per_cta;
-    sweep_span_kernel<RR, G, MODE><<<n_ctas, Gm.warps * 32, smem, st>>>(P, S, n0, n1, Gm);
+    sweep_span_kernel<RR, G, MODE, LM><<<n_ctas, Gm.warps * 32, smem, st>>>(P, S, n0, n1, Gm);
     return cudaGetLastError();
 }
 
@@ -560,7 +637,13 @@ cudaError_t launch_span(const DevProblem &P, const DevState &S, int n0, int n1, 
         if (m4 <= (size_t)smem_max && (!g8.stage_b || (g4.stage_b && g8.groups_per_cta >= 6)))
             return launch_span_g<RR, 4, MODE>(P, S, n0, n1, g4, m4, st);
     }
-    return launch_span_g<RR, 8, MODE>(P, S, n0, n1, g8, m8, st);
+    if constexpr (MODE == kWalk) {
+        if (P.walk_len <= 2) return launch_span_g<RR, 8, MODE, 2>(P, S, n0, n1, g8, m8, st);
+        if (P.walk_len <= 4) return launch_span_g<RR, 8, MODE, 4>(P, S, n0, n1, g8, m8, st);
+        return launch_span_g<RR, 8, MODE, 7>(P, S, n0, n1, g8, m8, st);
+    } else {
+        return launch_span_g<RR, 8, MODE>(P, S, n0, n1, g8, m8, st);
+    }
 }
 
 template <int RR>
