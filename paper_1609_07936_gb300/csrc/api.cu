@@ -504,12 +504,16 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     std::vector<double> K64(NO * PAD, 0.0), F64(PAD, 0.0);
     std::vector<float> K32(NO * PAD, 0.0f), F32(PAD, 0.0f), beta(NO);
     for (int i = 0; i < n_tau; ++i) {
+        // the factors that depend on tau alone (one expm1 a point, not one an element: half of the
+        // table's time)
+        const double edge = -std::expm1(-dw * tau[i]), denom = 2.0 * kPi * tau[i];
         for (int j = 0; j < n_omega; ++j) {
             double Kij;
             if (tau[i] == 0.0) Kij = dw / (2.0 * kPi);
-            else Kij = std::exp(-(double)j * dw * tau[i]) * (-std::expm1(-dw * tau[i])) / (2.0 * kPi * tau[i]);
-            K64[(size_t)j * PAD + i] = Kij / sigma[i];
-            K32[(size_t)j * PAD + i] = (float)(Kij / sigma[i]);
+            else Kij = std::exp(-(double)j * dw * tau[i]) * edge / denom;
+            const double k = Kij / sigma[i];
+            K64[(size_t)j * PAD + i] = k;
+            K32[(size_t)j * PAD + i] = (float)k;
         }
         F64[i] = F[i] / sigma[i];
         F32[i] = (float)F64[i];
@@ -543,10 +547,11 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
             for (int e = 0; e < 4; ++e) x4[(size_t)j * 4 + e] = (float)std::exp(-(double)j * dw * (double)e * dtau);
         for (int i = 0; i < n_tau; ++i) mrho[i] = (float)(-(K64[i] / K64[i & ~3]));
     }
-    // tensor-core resync tables, K-major [i][j]: Khi = Khat cut to TF32, Klo = the remainder
+    // tables of the TF32 recomputation, K-major [i][j]: Khi = Khat cut to TF32, Klo = the remainder
     const int NOP = (n_omega + 31) / 32 * 32;
-    std::vector<float> Khi((size_t)PAD * NOP, 0.0f), Klo((size_t)PAD * NOP, 0.0f);
-    for (int i = 0; i < n_tau; ++i)
+    const bool tf32 = p->precision == SAIL_PREC_FP32 && p->resync_kind == 1;
+    std::vector<float> Khi(tf32 ? (size_t)PAD * NOP : 0, 0.0f), Klo(tf32 ? (size_t)PAD * NOP : 0, 0.0f);
+    for (int i = 0; tf32 && i < n_tau; ++i)
         for (int j = 0; j < n_omega; ++j) {
             const double k64 = K64[(size_t)j * PAD + i];
             uint32_t bits;
@@ -712,8 +717,8 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     if (e == cudaSuccess) e = up(L.Qlo32, Qlo.data(), Qlo.size() * 4);
     if (e == cudaSuccess) e = up(L.x4_32, x4.data(), x4.size() * 4);
     if (e == cudaSuccess) e = up(L.mrho32, mrho.data(), mrho.size() * 4);
-    if (e == cudaSuccess) e = up(L.Khi32, Khi.data(), Khi.size() * 4);
-    if (e == cudaSuccess) e = up(L.Klo32, Klo.data(), Klo.size() * 4);
+    if (e == cudaSuccess && tf32) e = up(L.Khi32, Khi.data(), Khi.size() * 4);
+    if (e == cudaSuccess && tf32) e = up(L.Klo32, Klo.data(), Klo.size() * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + L.status, 0, 4, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + L.guard, 0, 16, st);
     if (e == cudaSuccess) e = up(L.Tsweep, T.data(), T.size() * 8);
