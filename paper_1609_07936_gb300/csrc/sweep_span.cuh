@@ -490,7 +490,8 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 const float ap = fmaf(r, ghi * bp, -cur.mdp);
                 const float as = fmaf(r, ghi * bs, -cur.mds);
                 const bool ok = ap >= 0.0f && as >= 0.0f;
-                pos += !ok;
+                // an index walk forms its amplitudes anew, also a null move's, whose threshold alone is negative
+                pos += WALK ? !ok && cur.thr > 0.0f : !ok;
                 float gah = ghi, gal = glo;
                 pair_scale(gah, gal, r);
                 const float inv_g = rcp_rn(gah);

@@ -55,6 +55,31 @@ def test_span_sweep_takes_the_decisions_of_the_sweep_over_tau(n_tau, n_omega, W,
     assert x[3].sum() > 0
 
 
+@pytest.mark.parametrize("n_omega,kw", [
+    (1001, {}), (1003, {"hastings": True}), (1006, {"index_walk_len": 2}), (1001, {"index_walk_len": 3}),
+    (1007, {"index_walk_len": 7, "walk_uniform": 0.2}), (1000, {"index_walk_len": 1}),
+])
+def test_a_restored_run_takes_the_decisions_of_the_sweep_over_tau(n_omega, kw):
+    """After set_state the residue is not known and a block of more than 625000 moves runs over tau; a
+    handle restored from that very state knows it and runs the span sweep.  Same spectra, accepted
+    moves and positivity rejections, also where the sweep ends inside a batch of draws."""
+    P = _problem(40, n_omega)
+    prm = sail.Params(n_walkers=301, n_sweeps=20000, sweeps_per_block=3, branching=False, A=P.A, B=P.B, seed=11,
+                      resync_kind=sail.RESYNC_FP32, **kw)
+    runs = []
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega, prm)
+    g.set_state(g.state()[0])
+    blob = g.checkpoint()
+    h = sail.Sail(P.tau, P.F, P.sigma, P.omega, prm)
+    h.restore(blob)
+    for s in (g, h):
+        stats = s.anneal(1)[0]
+        runs.append((*s.state()[:4], stats["positivity_rejected"], stats["acceptance"]))
+        s.close()
+    for u, v in zip(*runs):
+        np.testing.assert_array_equal(np.asarray(u), np.asarray(v))
+
+
 def test_wide_ranges_keep_the_sweep_over_tau():
     """tau up to 150 with noise falling as e^{-tau} to 1e-12: the columns need 36 directions, 32 leave 1.2e-7
     of one, and the sweep over tau serves the problem."""
