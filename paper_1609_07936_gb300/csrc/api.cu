@@ -64,6 +64,12 @@ constexpr double kPi = 3.14159265358979323846;
 // largest weighted model term (max Khat_ij * A) and weighted datum an FP32 state accepts: their
 // squares summed over 512 tau points stay below 1e33, far inside FP32's range
 constexpr double kFp32TermMax = 1e15;
+// Conversion buffer of an FP32 handle's state on its way from or to the host, at most (a smaller state takes
+// less): a copy costs ~10 us besides its bytes, 2 MB another 6 us.
+constexpr size_t kConvBytes = (size_t)2 << 20;
+// Arrays of fewer elements are converted by the host thread (0.23 ns an element), which needs no launch
+// before its copy (~4 us): a state of 20000 elements in and out 117 us against 129 on the device.
+constexpr size_t kConvMin = 32768;
 
 size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
@@ -77,6 +83,7 @@ struct Layout {
     size_t pr_walker, pr_p, pr_s, pr_eps, pr_delta, pr_ok;
     size_t tma_a, tma_b;     // pre-tiled BF16 pieces of the spectra and the kernel table (resync kind 2)
     size_t chi2_all;         // chi2 of the whole population (sail_branch_solve)
+    size_t conv, conv_bytes; // FP64 copy of a piece of the state on its way from or to the host (FP32)
     size_t Kspan, Uspan, Fspan, U64, span_worst;   // the kernel columns' basis (FP32, sweep_span.cuh)
     size_t total;
     int max_events;
@@ -144,7 +151,12 @@ Layout make_layout(int n_tau, int n_omega, const sail_params &p) {
     L.n_used = take(4);
     L.cut = take(8);
     L.avg_idx = take(W * 4);
-    if (p.precision == SAIL_PREC_FP32) L.avg_parts = take((size_t)2 * kAvgChunks * NO * 8);
+    if (p.precision == SAIL_PREC_FP32) {
+        // the parts of an average and the conversion buffer share one region (neither outlives its call)
+        L.conv_bytes = std::max((size_t)2 * kAvgChunks * NO * 8,
+                                std::min(kConvBytes, W * std::max(NO, (size_t)n_tau) * 8));
+        L.conv = L.avg_parts = take(L.conv_bytes);
+    }
     L.pr_walker = take((size_t)kProbeMax * 4);
     L.pr_p = take((size_t)kProbeMax * 4);
     L.pr_s = take((size_t)kProbeMax * 4);
@@ -794,6 +806,29 @@ int sail_get_info(sail_t h, sail_info *info) {
 
 namespace {
 
+// `total` elements of an FP32 state array (rows of cols, pitch apart) as FP64 on the host: converted on the
+// device a piece at a time, or here where there are few.
+int state_to_host(sail_t h, const float *src, int cols, int pitch, size_t total, double *out) {
+    if (total < kConvMin) {
+        const size_t rows = total / cols;
+        std::vector<float> f(rows * pitch);
+        SAIL_CUDA(cudaMemcpyAsync(f.data(), src, f.size() * 4, cudaMemcpyDeviceToHost, h->stream), "D2H");
+        SAIL_CUDA(cudaStreamSynchronize(h->stream), "D2H sync");
+        for (size_t w = 0; w < rows; ++w)
+            for (int i = 0; i < cols; ++i) out[w * cols + i] = (double)f[w * pitch + i];
+        return SAIL_OK;
+    }
+    double *buf = (double *)(h->ws + h->L.conv);
+    const size_t piece = h->L.conv_bytes / 8;
+    for (size_t q = 0; q < total; q += piece) {
+        const size_t n = std::min(piece, total - q);
+        SAIL_CUDA(launch_widen(src, cols, pitch, q, n, buf, h->stream), "state launch");
+        h->launches += 1;
+        SAIL_CUDA(cudaMemcpyAsync(out + q, buf, n * 8, cudaMemcpyDeviceToHost, h->stream), "D2H");
+    }
+    return SAIL_OK;
+}
+
 int average_to_host(sail_t h, double *mean, double *err, int *n_used, double *chi2_mean) {
     char *ws = h->ws;
     int l = 0;
@@ -1067,27 +1102,22 @@ int sail_get_state(sail_t h, double *a, double *R, double *chi2, int *acc_prev, 
     cudaStream_t st = h->stream;
     char *ws = h->ws;
     const bool f64 = h->prm.precision == SAIL_PREC_FP64;
-    std::vector<float> fbuf;
     std::vector<double> rbuf;
     if (a) {
         if (f64) SAIL_CUDA(cudaMemcpyAsync(a, ws + h->L.a64, W * NO * 8, cudaMemcpyDeviceToHost, st), "D2H");
-        else { fbuf.resize(W * NO); SAIL_CUDA(cudaMemcpyAsync(fbuf.data(), ws + h->L.b32, W * NO * 4, cudaMemcpyDeviceToHost, st), "D2H"); }
+        else if (const int rc = state_to_host(h, h->S.b32, (int)NO, (int)NO, W * NO, a)) return rc;
     }
-    std::vector<float> rf;
     if (R) {
         if (f64) { rbuf.resize(W * PAD); SAIL_CUDA(cudaMemcpyAsync(rbuf.data(), ws + h->L.R64, W * PAD * 8, cudaMemcpyDeviceToHost, st), "D2H"); }
-        else { rf.resize(W * PAD); SAIL_CUDA(cudaMemcpyAsync(rf.data(), ws + h->L.R32, W * PAD * 4, cudaMemcpyDeviceToHost, st), "D2H"); }
+        else if (const int rc = state_to_host(h, h->S.R32, h->n_tau, (int)PAD, W * h->n_tau, R)) return rc;
     }
     if (chi2) SAIL_CUDA(cudaMemcpyAsync(chi2, ws + h->L.chi2, W * 8, cudaMemcpyDeviceToHost, st), "D2H");
     if (acc_prev) SAIL_CUDA(cudaMemcpyAsync(acc_prev, ws + h->L.acc_prev, W * 4, cudaMemcpyDeviceToHost, st), "D2H");
     if (hash) SAIL_CUDA(cudaMemcpyAsync(hash, ws + h->L.hash, W * 8, cudaMemcpyDeviceToHost, st), "D2H");
     SAIL_CUDA(cudaStreamSynchronize(st), "get_state sync");
-    if (a && !f64) for (size_t q = 0; q < W * NO; ++q) a[q] = (double)fbuf[q];
-    if (R) {
+    if (R && f64)
         for (size_t w = 0; w < W; ++w)
-            for (int i = 0; i < h->n_tau; ++i)
-                R[w * h->n_tau + i] = f64 ? rbuf[w * PAD + i] : (double)rf[w * PAD + i];
-    }
+            for (int i = 0; i < h->n_tau; ++i) R[w * h->n_tau + i] = rbuf[w * PAD + i];
     return SAIL_OK;
 }
 
@@ -1096,16 +1126,26 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev) {
     const size_t W = (size_t)h->prm.n_walkers, NO = (size_t)h->n_omega;
     cudaStream_t st = h->stream;
     char *ws = h->ws;
-    std::vector<float> fbuf, g;
+    std::vector<float> fbuf;
     if (h->prm.precision == SAIL_PREC_FP64) {
         SAIL_CUDA(cudaMemcpyAsync(ws + h->L.a64, a, W * NO * 8, cudaMemcpyHostToDevice, st), "H2D");
     } else {
-        fbuf.resize(W * NO);
-        for (size_t q = 0; q < W * NO; ++q) fbuf[q] = (float)a[q];
-        g.resize(2 * W);
-        for (size_t w = 0; w < W; ++w) { g[2 * w] = 1.0f; g[2 * w + 1] = 0.0f; }
-        SAIL_CUDA(cudaMemcpyAsync(ws + h->L.b32, fbuf.data(), W * NO * 4, cudaMemcpyHostToDevice, st), "H2D");
-        SAIL_CUDA(cudaMemcpyAsync(ws + h->L.g2, g.data(), W * 2 * 4, cudaMemcpyHostToDevice, st), "H2D");
+        double *buf = (double *)(ws + h->L.conv);
+        const size_t piece = h->L.conv_bytes / 8;
+        if (W * NO < kConvMin) {
+            fbuf.resize(W * NO);
+            for (size_t q = 0; q < W * NO; ++q) fbuf[q] = (float)a[q];
+            SAIL_CUDA(cudaMemcpyAsync(h->S.b32, fbuf.data(), W * NO * 4, cudaMemcpyHostToDevice, st), "H2D");
+        } else {
+            for (size_t q = 0; q < W * NO; q += piece) {
+                const size_t n = std::min(piece, W * NO - q);
+                SAIL_CUDA(cudaMemcpyAsync(buf, a + q, n * 8, cudaMemcpyHostToDevice, st), "H2D");
+                SAIL_CUDA(launch_narrow(buf, n, h->S.b32 + q, st), "set_state launch");
+                h->launches += 1;
+            }
+        }
+        SAIL_CUDA(launch_unit_scale(h->prm.n_walkers, h->S.g2, st), "set_state launch");
+        h->launches += 1;
     }
     if (acc_prev) SAIL_CUDA(cudaMemcpyAsync(ws + h->L.acc_prev, acc_prev, W * 4, cudaMemcpyHostToDevice, st), "H2D");
     int l = 0;

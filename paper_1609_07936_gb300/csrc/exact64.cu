@@ -917,6 +917,28 @@ __global__ void walker_rows_kernel(DevProblem P, DevState S, int precision, cons
         R_rows[(size_t)q * NT + i] = precision == 0 ? S.R64[(size_t)l * PAD + i] : (double)S.R32[(size_t)l * PAD + i];
 }
 
+// Elements [q0, q0 + n) of an FP32 array of rows of `cols` (`pitch` apart) as FP64, and the way back (rows
+// without gaps): states cross to the host in FP64, and the conversion is bound by memory here, 3 us for
+// 512000 elements, where a host thread took 130 (in) to 230 us (out), page faults of its buffer included.
+// set_state and state of 1024 walkers x 500 bins x 200 tau: 0.66 -> 0.39 ms.
+__global__ void __launch_bounds__(256) widen_kernel(const float *src, int cols, int pitch, size_t q0, size_t n, double *out) {
+    const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const size_t at = q0 + q;
+    out[q] = (double)src[cols == pitch ? at : at / cols * pitch + at % cols];
+}
+__global__ void __launch_bounds__(256) narrow_kernel(const double *in, size_t n, float *dst) {
+    const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) dst[q] = (float)in[q];
+}
+// every walker's common scale = 1
+__global__ void __launch_bounds__(256) unit_scale_kernel(int n_walkers, float *g2) {
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= n_walkers) return;
+    g2[2 * w] = 1.0f;
+    g2[2 * w + 1] = 0.0f;
+}
+
 // Imprinting from donor rows (Sec. 2.5), the arithmetic of imprint_kernel with the donor's
 // values read from rows in this device's memory: walker idx[q] <- t row q + (1 - t) itself.
 __global__ void __launch_bounds__(128) imprint_rows_kernel(DevProblem P, DevState S, int precision, const int *idx,
@@ -1395,6 +1417,21 @@ cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const Br
 cudaError_t launch_walker_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,
                                double *a_rows, double *R_rows, cudaStream_t st) {
     walker_rows_kernel<<<n, 128, 0, st>>>(P, S, precision, idx, a_rows, R_rows);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_widen(const float *src, int cols, int pitch, size_t q0, size_t n, double *out, cudaStream_t st) {
+    widen_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, cols, pitch, q0, n, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_narrow(const double *in, size_t n, float *dst, cudaStream_t st) {
+    narrow_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, dst);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unit_scale(int n_walkers, float *g2, cudaStream_t st) {
+    unit_scale_kernel<<<(n_walkers + 255) / 256, 256, 0, st>>>(n_walkers, g2);
     return cudaGetLastError();
 }
 

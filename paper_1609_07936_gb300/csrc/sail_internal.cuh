@@ -171,6 +171,10 @@ cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const Br
 // Rows of walkers idx[0..n) (device array) in FP64, and imprinting of walkers idx from donor rows.
 cudaError_t launch_walker_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,
                                double *a_rows, double *R_rows, cudaStream_t st);
+// Elements [q0, q0 + n) of an FP32 array (rows of cols, pitch apart) to FP64; FP64 to FP32; scales to 1.
+cudaError_t launch_widen(const float *src, int cols, int pitch, size_t q0, size_t n, double *out, cudaStream_t st);
+cudaError_t launch_narrow(const double *in, size_t n, float *dst, cudaStream_t st);
+cudaError_t launch_unit_scale(int n_walkers, float *g2, cudaStream_t st);
 cudaError_t launch_imprint_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,
                                 const double *a_rows, const double *R_rows, double t, cudaStream_t st);
 // Smoothing (Sec. smoothing) of every walker's spectrum with strength s and the tilt that
