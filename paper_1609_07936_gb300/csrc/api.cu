@@ -302,7 +302,8 @@ int sweep_ahead_next(const sail_ctx *h) {
 // between two recomputations) relative to the magnitude of its terms, S = eps_max |R| (|R| + |Fhat|)
 // that magnitude.  Measured on the paper-scale problem, walkers of 4096 that parted in a block of
 // 4.1e8 moves: 0 at T = 10 chi2_0 .. 0.5 chi2_0 (estimate 0.004 .. 0.06), 7 to 17 at T = 1e6 near
-// equilibrium (estimate 16); the line is drawn at 1/16 of a decision a block.
+// equilibrium (estimate 16).  The line lies at 1/64 of a decision a block: at 1/16, 3 of 6 runs of the band
+// example (estimate 0.016 a block) parted from the sweep over tau within 6 blocks and 1 of 60 tiny inversions.
 bool span_next(const sail_ctx *h, int n0, int n1) {
     const sail_params &p = h->prm;
     if (h->P.span == 0 || p.shared_bins > 1 || p.fp64_accept) return false;
@@ -310,7 +311,7 @@ bool span_next(const sail_ctx *h, int n0, int n1) {
     const double eps = p.move_scale > 0.0 ? p.move_scale : 1.0 / h->n_omega;
     const double R = std::sqrt(h->chi2_ref), S = eps * R * (R + h->F_norm);
     const double moves = (double)(n1 - n0) * p.n_walkers * h->n_omega;
-    return moves * 1e-7 * std::min(1.0, S / T) <= 0.0625;     // chi2 not known (NaN): S / T counts as 1
+    return moves * 1e-7 * std::min(1.0, S / T) <= 0.015625;     // chi2 not known (NaN): S / T counts as 1
 }
 
 // A named NVTX range around the host calls that enqueue one phase of the schedule (sweep,
@@ -1126,7 +1127,7 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev) {
     const size_t W = (size_t)h->prm.n_walkers, NO = (size_t)h->n_omega;
     cudaStream_t st = h->stream;
     char *ws = h->ws;
-    std::vector<float> fbuf;
+    std::vector<float> fbuf, g;
     if (h->prm.precision == SAIL_PREC_FP64) {
         SAIL_CUDA(cudaMemcpyAsync(ws + h->L.a64, a, W * NO * 8, cudaMemcpyHostToDevice, st), "H2D");
     } else {
@@ -1134,8 +1135,11 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev) {
         const size_t piece = h->L.conv_bytes / 8;
         if (W * NO < kConvMin) {
             fbuf.resize(W * NO);
+            g.resize(2 * W);
             for (size_t q = 0; q < W * NO; ++q) fbuf[q] = (float)a[q];
+            for (size_t w = 0; w < W; ++w) { g[2 * w] = 1.0f; g[2 * w + 1] = 0.0f; }
             SAIL_CUDA(cudaMemcpyAsync(h->S.b32, fbuf.data(), W * NO * 4, cudaMemcpyHostToDevice, st), "H2D");
+            SAIL_CUDA(cudaMemcpyAsync(h->S.g2, g.data(), W * 2 * 4, cudaMemcpyHostToDevice, st), "H2D");
         } else {
             for (size_t q = 0; q < W * NO; q += piece) {
                 const size_t n = std::min(piece, W * NO - q);
@@ -1143,9 +1147,9 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev) {
                 SAIL_CUDA(launch_narrow(buf, n, h->S.b32 + q, st), "set_state launch");
                 h->launches += 1;
             }
+            SAIL_CUDA(launch_unit_scale(h->prm.n_walkers, h->S.g2, st), "set_state launch");
+            h->launches += 1;
         }
-        SAIL_CUDA(launch_unit_scale(h->prm.n_walkers, h->S.g2, st), "set_state launch");
-        h->launches += 1;
     }
     if (acc_prev) SAIL_CUDA(cudaMemcpyAsync(ws + h->L.acc_prev, acc_prev, W * 4, cudaMemcpyHostToDevice, st), "H2D");
     int l = 0;

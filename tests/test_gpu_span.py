@@ -60,7 +60,7 @@ def test_span_sweep_takes_the_decisions_of_the_sweep_over_tau(n_tau, n_omega, W,
     (1007, {"index_walk_len": 7, "walk_uniform": 0.2}), (1000, {"index_walk_len": 1}),
 ])
 def test_a_restored_run_takes_the_decisions_of_the_sweep_over_tau(n_omega, kw):
-    """After set_state the residue is not known and a block of more than 625000 moves runs over tau; a
+    """After set_state the residue is not known and a block of more than 156250 moves runs over tau; a
     handle restored from that very state knows it and runs the span sweep.  Same spectra, accepted
     moves and positivity rejections, also where the sweep ends inside a batch of draws."""
     P = _problem(40, n_omega)
