@@ -588,12 +588,6 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
             return b[j];
         }
     };
-    auto bset = [&](int j, float v) {
-        if constexpr (STAGED)
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(bsh + 4u * (uint32_t)j), "f"(v) : "memory");
-        else
-            b[j] = v;
-    };
 
     f2 R[C][H], M[C][H];
 #pragma unroll
@@ -734,7 +728,9 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
                     acc_k = ok && (MODE == kHastings ? D < cur.thr : (D <= 0.0f || D < cur.thr));
                 }
                 // the update, branch-free: a mask of 1 or 0 adds d or leaves R and M as they are, and every
-                // lane of the walker stores the same two values (each later reads its own store)
+                // lane of the walker stores the same two values (each later reads its own store).  The
+                // barrier orders the lanes' stores of consecutive moves, and their reads of this move
+                // before its stores
                 const float am = acc_k ? 1.0f : 0.0f;
                 const f2 am2 = pk(am, am), nam2 = pk(-am, -am);
 #pragma unroll
@@ -749,6 +745,7 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
                 pair_scale(gah, gal, r);
                 const float inv_g = rcp_rn(gah);
                 const float bp_new = ap * inv_g, bs_new = as * inv_g;
+                __syncwarp();
                 put_if<STAGED>(am, b, p, s, bp_new, bs_new);
                 if constexpr (BAHEAD) {
                     const int pn = nxt.ps & 0xFFFF, sn = nxt.ps >> 16;
@@ -773,6 +770,7 @@ __device__ __forceinline__ void run_group(const DevProblem &P, const DevState &S
         npos += pos;
         if (active && S.acc_trace && gl == 0) S.acc_trace[(size_t)n * P.n_walkers + w] = acc;
     }
+    __syncwarp();                      // the lanes' writes of b, before other lanes fold them
     if (!active) return;
     // fold the common scale into the spectrum and write the walker back
     float *bg = S.b32 + (size_t)w * NO;

@@ -319,7 +319,8 @@ __device__ __forceinline__ void span_write_back(const DevProblem &P, const DevSt
 //          those bins (until the batch turns over the replacement waits apart, so that nothing
 //          waits for the read), and hands them over by shuffle
 // Every lane of a walker writes an accepted move's two amplitudes (the same values), so each
-// lane later reads its own write and the loop needs no barrier.
+// lane later reads its own write.  The warp barrier before the write orders it against the other
+// lanes' reads of the same move and their writes of the move before, whose shuffles order no memory.
 //
 // LM > 0 (index walk): the walk's steps unrolled to LM >= P.walk_len.  The proposals of a walk do not
 // depend on the state, so the steps' words are drawn and handed out one move ahead, and b at all of
@@ -503,6 +504,7 @@ __device__ __forceinline__ void run_span(const DevProblem &P, const DevState &S,
                 const f2 am2 = pk(am, am);
 #pragma unroll
                 for (int u = 0; u < NV; ++u) span_add<RR>(R[u], C[u], d[u], am, am2, minus_one);
+                __syncwarp();          // orders the lanes' stores of b (see above)
                 put_if<STAGED>(am, b, p, s, ap_b, as_b);
                 ghi = acc_k ? gah : ghi;
                 glo = acc_k ? gal : glo;
