@@ -1521,14 +1521,13 @@ int batch_class(const DevProblem &P) {
 
 // Shared memory that a problem may ask of its classes' kernels (it changes between the sweep over
 // tau and the span sweep from block to block).
-void batch_reserve(size_t *smem, const DevProblem &P) {
-    int dev = 0, smem_max = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+cudaError_t batch_reserve(size_t *smem, const DevProblem &P) {
     const int mode = sweep_mode(P);
-    size_t &tau = smem[3 * (P.lanes == 8 ? 1 : 0) + mode], &span = smem[6 + mode];
+    size_t &tau = smem[3 * (P.lanes == 8 ? 1 : 0) + mode], &span = smem[6 + mode], bytes = 0;
     tau = std::max(tau, sweep_fp32_table_bytes(P));
-    if (P.span > 0) span = std::max(span, span_batch_smem(P, smem_max));
+    const cudaError_t e = P.span > 0 ? span_batch_smem(P, mode, &bytes) : cudaSuccess;
+    span = std::max(span, bytes);
+    return e;
 }
 
 void batch_streams_create(sail_batch_ctx *b) {
@@ -1640,7 +1639,12 @@ int sail_batch_create(sail_batch_t *out, int n, const sail_problem *probs, int a
             return rc;
         }
         b->h.push_back(h);
-        batch_reserve(b->smem, h->P);
+        const cudaError_t e = batch_reserve(b->smem, h->P);
+        if (e != cudaSuccess) {
+            for (sail_t x : b->h) sail_destroy(x);
+            delete b;
+            return cuda_fail(e, "batch kernel attributes");
+        }
         off += align_up(sub);
     }
     b->autotune = autotune;
@@ -1964,8 +1968,15 @@ int server_step(sail_server_t s, int *completed, int max_completed, int *n_compl
             s->queue.pop_front();
         }
         sail_t h = nullptr;
-        const int rc = sail_create(&h, r.tau.data(), r.F.data(), r.sigma.data(), (int)r.tau.size(), r.omega.data(),
+        int rc = sail_create(&h, r.tau.data(), r.F.data(), r.sigma.data(), (int)r.tau.size(), r.omega.data(),
                                    (int)r.omega.size(), &r.params, b.ws + off, r.bytes, b.stream);
+        if (rc == SAIL_OK) {
+            const cudaError_t e = batch_reserve(b.smem, h->P);
+            if (e != cudaSuccess) {
+                sail_destroy(h);
+                rc = cuda_fail(e, "batch kernel attributes");
+            }
+        }
         if (rc) {
             region_give(s, off, r.bytes);
             std::lock_guard<std::mutex> lk(s->mu);
@@ -1977,7 +1988,6 @@ int server_step(sail_server_t s, int *completed, int max_completed, int *n_compl
             return rc;
         }
         b.h[slot] = h;
-        batch_reserve(b.smem, h->P);
         s->slot_off[slot] = off;
         s->slot_size[slot] = r.bytes;
         s->slot_id[slot] = r.id;

@@ -217,9 +217,10 @@ cudaError_t launch_sweep_batch(const BatchProblem *d_probs, const BatchItem *d_i
 cudaError_t launch_sweep_batch8(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                 size_t smem, int warps, int mode, cudaStream_t st);
 // The batched span sweep of problems whose P.span_on is set (any widths together): blocks of `warps`
-// warps (at most 16), smem at least the problems' span_batch_smem; lanes per walker by mode (the
-// results do not depend on it).
-size_t span_batch_smem(const DevProblem &P, int smem_max);
+// warps (at most 16), smem at least the problems' span_batch_smem (which leaves room for what the
+// kernel of that move-loop mode holds besides); lanes per walker by mode (the results do not depend
+// on it).
+cudaError_t span_batch_smem(const DevProblem &P, int mode, size_t *bytes);
 inline int span_batch_lanes(int mode) { return mode == 0 ? 4 : 8; }
 cudaError_t launch_span_batch(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                               size_t smem, int warps, int mode, cudaStream_t st);

@@ -702,6 +702,16 @@ __global__ void __launch_bounds__(32 * kSpanWarps, 1) sweep_span_batch_kernel(co
     }
 }
 
+// Shared memory the kernel holds besides the launch's: the two together must stay within the device's
+// limit per block.
+template <int G, int MODE>
+cudaError_t span_batch_static(size_t *bytes) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, sweep_span_batch_kernel<G, MODE>);
+    *bytes = e == cudaSuccess ? a.sharedSizeBytes : 0;
+    return e;
+}
+
 template <int G, int MODE>
 cudaError_t launch_span_batch_g(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                 size_t smem, int warps, cudaStream_t st) {

@@ -7,10 +7,19 @@ namespace sail {
 cudaError_t launch_span_batch_modes(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                     size_t smem, int warps, int mode, cudaStream_t st);
 
-size_t span_batch_smem(const DevProblem &P, int smem_max) {
+cudaError_t span_batch_static_modes(int mode, size_t *bytes);
+
+cudaError_t span_batch_smem(const DevProblem &P, int mode, size_t *bytes) {
+    int dev = 0, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    size_t fixed = 0;
+    const cudaError_t e = mode == kPlain ? span_batch_static<4, kPlain>(&fixed) : span_batch_static_modes(mode, &fixed);
+    if (e != cudaSuccess) return e;
     const size_t base = span_ring_bytes(kSpanWarps) + (size_t)span_vec_floats(P.n_omega) * 4;
     const size_t all = base + (size_t)P.n_omega * P.span * 4;
-    return all <= (size_t)smem_max ? all : base;
+    *bytes = all + fixed <= (size_t)smem_max ? all : base;
+    return cudaSuccess;
 }
 
 cudaError_t launch_span_batch(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter, size_t smem,

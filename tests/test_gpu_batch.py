@@ -125,3 +125,26 @@ def test_batch_takes_the_oracle_decisions():
             np.testing.assert_allclose(a[w], an.a[w], rtol=0, atol=1e-4 * an.a[w].max())
     assert lanes == {8, 16}
     batch.close()
+
+
+@pytest.mark.parametrize("kw", [{}, {"hastings": True}, {"index_walk_len": 2}])
+def test_a_column_table_at_the_limit_of_shared_memory(kw):
+    """1920 bins with 24 basis directions: rings, vectors and column table together are the device's
+    227 KB a block to the byte, which the batched kernel shares with a word of its own.  The batch
+    runs and its problems end as they do alone."""
+    probs = []
+    for k, (nt, no, nw) in enumerate([(200, 1920, 70), (40, 37, 33)]):
+        tau = 8.0 * np.arange(nt, dtype=np.float64) / (nt - 1)
+        P = make_problem(f"limit{k}", tau, no, 20.0, [Peak("lorentz", 2.0, 0.3, 0.6), Peak("lorentz", 5.0, 0.5, 0.4)], 1e-4, 3, nw)
+        prm = sail.Params(n_walkers=nw, n_sweeps=20000, sweeps_per_block=3, resync_every=2, branching=False, A=P.A, B=P.B,
+                          seed=70 + k, resync_kind=sail.RESYNC_FP32, **kw)
+        probs.append((P, prm))
+    batch = sail.Batch([(P.tau, P.F, P.sigma, P.omega, prm) for P, prm in probs], autotune=False)
+    batch.anneal(1)
+    for h, (P, prm) in zip(batch.handles, probs):
+        alone = sail.Sail(P.tau, P.F, P.sigma, P.omega, prm)
+        alone.anneal(1)
+        for x, y in zip(h.state()[:4], alone.state()[:4]):
+            np.testing.assert_array_equal(x, y)
+        alone.close()
+    batch.close()
