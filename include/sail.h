@@ -203,7 +203,8 @@ typedef struct sail_info {
     long long sweep_launches, resync_launches, branch_launches;
     long long moves;           /* walker-moves proposed so far */
     int sweep_lanes;           /* FP32 sweep: GPU lanes per walker in use (0 for FP64) */
-    int sweep_ahead;           /* FP32 sweep: 1 if the next block runs the look-ahead move loop */
+    int sweep_ahead;           /* FP32 sweep: 1 if the next block, where it sweeps over tau, runs the
+                                  look-ahead move loop (sail_span_info: which blocks do not) */
     long long fp64_rechecks;   /* fp64_accept: decisions taken again in FP64 so far */
     long long fp64_flips;      /* ... of which the FP64 decision differed from the FP32 one */
 } sail_info;
@@ -253,6 +254,13 @@ int sail_anneal(sail_t h, int max_blocks, sail_block_stats *stats, int *n_done);
 int sail_average(sail_t h, double *S_mean, double *S_err, int *n_used, double *chi2_of_mean);
 
 int sail_get_info(sail_t h, sail_info *info);
+
+/*
+ * The sweep in the basis of the kernel's columns (sail_params.sweep_loop): *width receives the
+ * number of its directions (16, 24 or 32; 0: the handle's blocks all sweep over tau) and *blocks
+ * the number of blocks this handle has run in it so far (either may be NULL).
+ */
+int sail_span_info(sail_t h, int *width, int *blocks);
 
 /*
  * Copies walker state to host arrays (any may be NULL): a[n_walkers * n_omega] spectra

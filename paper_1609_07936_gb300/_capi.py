@@ -44,7 +44,7 @@ EXPORTS = [
     "sail_server_result", "sail_server_destroy", "sail_destroy", "sail_last_error",
     "sail_server_start", "sail_server_poll", "sail_server_stop", "sail_server_request_info", "sail_server_trace",
     "sail_checkpoint_size", "sail_checkpoint", "sail_restore",
-    "sail_branch_solve", "sail_walker_rows", "sail_imprint_rows",
+    "sail_branch_solve", "sail_walker_rows", "sail_imprint_rows", "sail_span_info",
 ]
 
 
@@ -137,6 +137,7 @@ def load(path: str = LIB_PATH):
     L.sail_anneal.argtypes = [vp, ctypes.c_int, ctypes.POINTER(CBlockStats), _ip]
     L.sail_average.argtypes = [vp, _dp, _dp, _ip, _dp]
     L.sail_get_info.argtypes = [vp, ctypes.POINTER(CInfo)]
+    L.sail_span_info.argtypes = [vp, _ip, _ip]
     L.sail_get_state.argtypes = [vp, _dp, _dp, _dp, _ip, _u64p]
     L.sail_set_state.argtypes = [vp, _dp, _ip]
     L.sail_get_trace.argtypes = [vp, _ip, _ip, _dp, _ip]
@@ -316,6 +317,12 @@ class Sail:
         ci = CInfo()
         _check(self.lib.sail_get_info(self._h, ctypes.byref(ci)))
         return {f[0]: getattr(ci, f[0]) for f in CInfo._fields_}
+
+    def span_info(self) -> dict:
+        """Directions of the kernel columns' basis (0: none) and the blocks swept in it so far."""
+        width, blocks = ctypes.c_int(0), ctypes.c_int(0)
+        _check(self.lib.sail_span_info(self._h, ctypes.byref(width), ctypes.byref(blocks)))
+        return {"width": width.value, "blocks": blocks.value}
 
     def anneal(self, max_blocks: int = 1 << 30) -> List[dict]:
         """Runs up to max_blocks blocks; returns one stats dict per block run."""

@@ -264,6 +264,7 @@ struct sail_ctx {
     int *status;             // device status word: nonzero after a timed-out device wait
     bool ahead_auto;         // FP32 sweep_loop 0 with enough walkers: the loop follows the rejections
     double pos_frac_last = -1.0;   // positivity-rejected share of the last block's proposals
+    int span_blocks = 0;     // blocks run in the span of the kernel's columns
     double chi2_ref;         // mean chi2 of the walkers before the next block (NaN: not known)
     double F_norm;           // |F / sigma|
     bool converged;          // chi2 of the averaged spectrum reached target_chi2
@@ -805,6 +806,13 @@ int sail_get_info(sail_t h, sail_info *info) {
     return SAIL_OK;
 }
 
+int sail_span_info(sail_t h, int *width, int *blocks) {
+    if (!h) return fail(SAIL_EINVAL, "NULL handle");
+    if (width) *width = h->P.span;
+    if (blocks) *blocks = h->span_blocks;
+    return SAIL_OK;
+}
+
 namespace {
 
 // `total` elements of an FP32 state array (rows of cols, pitch apart) as FP64 on the host: converted on the
@@ -1034,6 +1042,7 @@ int block_finish(sail_ctx *h, const BlockPending &b, sail_block_stats *out) {
     h->acc_seen = b.bc.acc;
     h->pos_seen = b.bc.pos;
     h->blocks_done += 1;
+    h->span_blocks += h->P.span_on != 0;
     if (p.target_chi2 > 0) {
         double c2 = 0;
         const int rc = average_to_host(h, nullptr, nullptr, nullptr, &c2);

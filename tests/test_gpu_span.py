@@ -95,3 +95,56 @@ def test_wide_ranges_keep_the_sweep_over_tau():
         out.append(g.state()[0])
         g.close()
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("n_tau,n_omega,W,tau_max,floor,width", [
+    (1, 8, 1, 8.0, 0.0, 16), (5, 3, 5, 8.0, 0.0, 16), (32, 64, 64, 2.0, 0.0, 16), (33, 65, 4097, 4.0, 0.0, 24),
+    (200, 1000, 63, 8.0, 0.0, 24), (200, 1001, 10001, 8.0, 0.0, 24), (512, 2043, 130, 8.0, 0.0, 24),
+    (96, 2600, 70, 8.0, 0.0, 24), (300, 501, 77, 40.0, 1e-3, 32),
+])
+@pytest.mark.parametrize("guard", [0, 1])
+def test_which_sweep_a_block_runs(n_tau, n_omega, W, tau_max, floor, width, guard):
+    """The widths of the bases (the numerical ranks of these kernels at 2^-26, in numpy: 1, 3, 15, 18, 23,
+    23, 23, 22 and 29) and, of the two sides that the comparison above takes, that one sweeps in the
+    basis and the other over tau."""
+    P = _problem(n_tau, n_omega, tau_max, floor)
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega,
+                  sail.Params(n_walkers=W, n_sweeps=20000, sweeps_per_block=3, resync_every=2, branching=False, A=P.A, B=P.B,
+                              seed=11, resync_kind=sail.RESYNC_FP32, fp64_accept=guard))
+    assert g.span_info()["blocks"] == 0
+    g.anneal(2)
+    assert g.span_info()["blocks"] == (0 if guard else 2)
+    if not guard:
+        assert g.span_info()["width"] == width
+    g.close()
+
+
+def test_wide_ranges_have_no_basis():
+    """The problem of the test above whose columns need 36 directions."""
+    tau = 150.0 * (np.arange(400, dtype=np.float64) / 399) ** 1.5
+    P = make_problem("wide", tau, 400, 20.0, [Peak("lorentz", 2.0, 0.3, 1.0)], 1e-4, 3, 1, noise_floor=1e-3)
+    sigma = 1e-2 * np.maximum(np.exp(-tau), 1e-12)
+    prm = sail.Params(n_walkers=40, n_sweeps=20000, sweeps_per_block=3, resync_every=2, branching=False, A=P.A, B=P.B, seed=5)
+    g = sail.Sail(P.tau, P.F_exact, sigma, P.omega, prm)
+    g.anneal(1)
+    assert g.span_info() == {"width": 0, "blocks": 0}
+    g.close()
+
+
+@pytest.mark.parametrize("kw", [{}, {"hastings": True}, {"index_walk_len": 2}, {"index_walk_len": 5}])
+def test_batched_span_sweep_ends_as_the_problem_alone(kw):
+    """Three widths in one batch, an odd number of walkers and sweeps that end inside a batch of draws."""
+    probs = [(_problem(32, 61, 2.0), 16), (_problem(200, 503), 24), (_problem(300, 501, 40.0, 1e-3), 32)]
+    prm = [sail.Params(n_walkers=61 + k, n_sweeps=20000, sweeps_per_block=3, resync_every=2, branching=False, A=P.A, B=P.B,
+                       seed=80 + k, resync_kind=sail.RESYNC_FP32, **kw) for k, (P, _) in enumerate(probs)]
+    batch = sail.Batch([(P.tau, P.F, P.sigma, P.omega, p) for (P, _), p in zip(probs, prm)], autotune=False)
+    batch.anneal(2)
+    for h, (P, width), p in zip(batch.handles, probs, prm):
+        assert h.span_info() == {"width": width, "blocks": 2}
+        alone = sail.Sail(P.tau, P.F, P.sigma, P.omega, p)
+        alone.anneal(2)
+        assert alone.span_info()["blocks"] == 2
+        for x, y in zip(h.state()[:4], alone.state()[:4]):
+            np.testing.assert_array_equal(x, y)
+        alone.close()
+    batch.close()
