@@ -92,7 +92,8 @@ typedef struct sail_params {
                                <= 256 on a uniform grid only: sail_create returns SAIL_EINVAL
                                otherwise; its one-move loop forms the kernel columns from
                                tables of every fourth tau point) or 16.  The choice sets the
-                               order of the FP32 delta-chi2 sum, so trajectories depend on it */
+                               order of the FP32 delta-chi2 sum, so trajectories depend on it; 8 or
+                               16 given, every block sweeps over tau (see sweep_loop) */
     /* The paper's protocol against the sawtooth instability (Sec. self-cooling, Sec. 2.5,
      * Sec. smoothing).  All three act at the end of every full block of k sweeps, in this
      * order: block statistics (acceptance; mean and smallest residue after the block's
@@ -147,11 +148,13 @@ typedef struct sail_params {
                                look-ahead's in the last bits); 0 = choose: look-ahead when the problem has
                                at least 16 walkers per SM (measured faster there, slower with fewer)
                                and the last block rejected at least 30% of its proposals for
-                               positivity (measured +12% at 40%, -6% at 22-27%).  Own-bin blocks in
-                               which no decision is expected within FP32's rounding of its
-                               threshold run a third loop whatever lanes and loop are chosen: the
-                               same draws and decisions, delta chi2 summed in an orthonormal basis
-                               of the kernel's columns (16 to 32 terms instead of n_tau) */
+                               positivity (measured +12% at 40%, -6% at 22-27%).  Where neither
+                               sweep_loop nor sweep_lanes is given, own-bin blocks in which no
+                               decision is expected within FP32's rounding of its threshold run a
+                               third loop: the same draws, delta chi2 summed in an orthonormal basis
+                               of the kernel's columns (16 to 32 terms instead of n_tau), so the same
+                               decisions but for those within that rounding (sail_span_info tells
+                               which blocks did) */
     double T_start_abs;     /* > 0: the geometric schedule starts at this absolute temperature
                                instead of T_start chi2_0 (skip the boiling far above the data's
                                scale, whatever chi2_0 is); 0 = T_start */

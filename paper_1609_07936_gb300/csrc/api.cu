@@ -294,6 +294,12 @@ int sweep_ahead_next(const sail_ctx *h) {
     return h->P.ahead;
 }
 
+// Whether a handle's blocks may run in the span of the kernel's columns at all: own bins, FP32
+// decisions, and neither the loop over tau nor its lanes (the order of its sums) asked for.
+bool span_allowed(const sail_params &p) {
+    return p.precision == SAIL_PREC_FP32 && p.shared_bins <= 1 && p.fp64_accept == 0 && p.sweep_loop == 0 && p.sweep_lanes == 0;
+}
+
 // Whether the next block's sweeps [n0, n1) run in the span of the kernel's columns
 // (sweep_span.cuh) or over tau.  The two round delta chi2 differently, and a decision that lies
 // within that rounding of its threshold can come out differently; at a low temperature one such
@@ -307,7 +313,7 @@ int sweep_ahead_next(const sail_ctx *h) {
 // example (estimate 0.016 a block) parted from the sweep over tau within 6 blocks and 1 of 60 tiny inversions.
 bool span_next(const sail_ctx *h, int n0, int n1) {
     const sail_params &p = h->prm;
-    if (h->P.span == 0 || p.shared_bins > 1 || p.fp64_accept) return false;
+    if (h->P.span == 0) return false;
     const double T = std::min(h->T[n0], h->T[n1 - 1]);
     const double eps = p.move_scale > 0.0 ? p.move_scale : 1.0 / h->n_omega;
     const double R = std::sqrt(h->chi2_ref), S = eps * R * (R + h->F_norm);
@@ -748,7 +754,7 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     if (e == cudaSuccess)
         e = launch_init_state(P, S, p->precision, (const double *)(ws + L.a0), (const double *)(ws + L.R0), chi2_0, st);
     h->launches = 1;
-    if (e == cudaSuccess && p->precision == SAIL_PREC_FP32) e = span_init(h, K64, F64);
+    if (e == cudaSuccess && span_allowed(*p)) e = span_init(h, K64, F64);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         delete h;
@@ -1072,7 +1078,7 @@ int sail_anneal(sail_t h, int max_blocks, sail_block_stats *stats, int *n_done) 
         BlockPending b{};
         b.n_begin = h->sweeps_done;
         b.block_end = block_end_of(h);
-        h->P.span_on = p.precision == SAIL_PREC_FP32 && span_next(h, b.n_begin, b.block_end);
+        h->P.span_on = span_next(h, b.n_begin, b.block_end);
         for (int n = b.n_begin; n < b.block_end;) {
             const int next = next_resync(h, n, b.block_end);
             const int tk = timed_begin(h);
