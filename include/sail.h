@@ -296,6 +296,15 @@ int sail_set_state(sail_t h, const double *a, const int *acc_prev);
  */
 int sail_branch_solve(sail_t h, int n_total, const double *chi2_all, int block, double fraction, int *m,
                       double *delta, int *zero_l, int *donor_l, int *n_pairs);
+
+/*
+ * Tells a shard the whole population's chi2 before its next block (host array in index order, n_total
+ * = walker_total): the choice of a block's sweep (sail_params.sweep_loop) follows the population's
+ * moves and mean residue, so that a shard chooses as the whole population in one handle does.  To be
+ * called before every block, after imprinting, with what every shard's sail_get_state gives; a shard
+ * that is not told sweeps all but its smallest blocks over tau.  *mean (may be NULL) receives the mean.
+ */
+int sail_population_residue(sail_t h, int n_total, const double *chi2_all, double *mean);
 int sail_walker_rows(sail_t h, int n, const int *idx, double *d_a_rows, double *d_R_rows);
 int sail_imprint_rows(sail_t h, int n, const int *idx, const double *d_a_rows, const double *d_R_rows, double t);
 

@@ -45,6 +45,7 @@ EXPORTS = [
     "sail_server_start", "sail_server_poll", "sail_server_stop", "sail_server_request_info", "sail_server_trace",
     "sail_checkpoint_size", "sail_checkpoint", "sail_restore",
     "sail_branch_solve", "sail_walker_rows", "sail_imprint_rows", "sail_span_info",
+    "sail_population_residue",
 ]
 
 
@@ -142,6 +143,7 @@ def load(path: str = LIB_PATH):
     L.sail_set_state.argtypes = [vp, _dp, _ip]
     L.sail_get_trace.argtypes = [vp, _ip, _ip, _dp, _ip]
     L.sail_branch_solve.argtypes = [vp, ctypes.c_int, _dp, ctypes.c_int, ctypes.c_double, _ip, _dp, _ip, _ip, _ip]
+    L.sail_population_residue.argtypes = [vp, ctypes.c_int, _dp, _dp]
     L.sail_walker_rows.argtypes = [vp, ctypes.c_int, _ip, vp, vp]
     L.sail_imprint_rows.argtypes = [vp, ctypes.c_int, _ip, vp, vp, ctypes.c_double]
     L.sail_checkpoint_size.argtypes = [vp, ctypes.POINTER(ctypes.c_size_t)]
@@ -388,6 +390,13 @@ class Sail:
         _check(self.lib.sail_branch_solve(self._h, n, _ptr(c), int(block), float(fraction), _ptr(m, _ip),
                                           ctypes.byref(delta), _ptr(zl, _ip), _ptr(dl, _ip), ctypes.byref(npairs)))
         return m, delta.value, zl[: npairs.value].copy(), dl[: npairs.value].copy()
+
+    def population_residue(self, chi2_all) -> float:
+        """Tells a shard the population's chi2 before its next block (sail_population_residue); their mean."""
+        c = _f64(chi2_all)
+        mean = ctypes.c_double(0)
+        _check(self.lib.sail_population_residue(self._h, c.size, _ptr(c), ctypes.byref(mean)))
+        return mean.value
 
     def walker_rows(self, idx):
         """Spectra and residuals of this handle's walkers idx, as FP64 device tensors."""

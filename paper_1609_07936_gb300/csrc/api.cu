@@ -265,7 +265,7 @@ struct sail_ctx {
     bool ahead_auto;         // FP32 sweep_loop 0 with enough walkers: the loop follows the rejections
     double pos_frac_last = -1.0;   // positivity-rejected share of the last block's proposals
     int span_blocks = 0;     // blocks run in the span of the kernel's columns
-    double chi2_ref;         // mean chi2 of the walkers before the next block (NaN: not known)
+    double chi2_ref;         // mean chi2 of the population before the next block (NaN: not known)
     double F_norm;           // |F / sigma|
     bool converged;          // chi2 of the averaged spectrum reached target_chi2
     double chi2_of_mean;
@@ -294,6 +294,35 @@ int sweep_ahead_next(const sail_ctx *h) {
     return h->P.ahead;
 }
 
+// Walkers of the population that the handle's walkers are part of.
+int population(const sail_ctx *h) { return std::max(h->prm.n_walkers, h->prm.walker_total); }
+
+// Mean of n chi2 values, added in the order of block_stats_kernel (the same bits as its sum).
+double mean_residue(const double *chi2, int n) {
+    std::vector<double> part(1024, 0.0);
+    for (int w = 0; w < n; ++w) part[w & 1023] += chi2[w];
+    double sum = 0.0;
+    for (int k = 0; k < 32; ++k) {
+        double v[32];
+        std::copy(part.begin() + 32 * k, part.begin() + 32 * k + 32, v);
+        for (int o = 16; o > 0; o >>= 1)
+            for (int l = 0; l < o; ++l) v[l] += v[l + o];
+        sum = k ? sum + v[0] : v[0];
+    }
+    return sum / n;
+}
+
+// Before a block: the mean residue, if the state came from outside since the last one.  A shard's is told
+// (sail_population_residue) or stays unknown.
+cudaError_t ref_update(sail_ctx *h) {
+    if (h->P.span == 0 || h->chi2_ref == h->chi2_ref || population(h) > h->prm.n_walkers) return cudaSuccess;
+    std::vector<double> chi2(h->prm.n_walkers);
+    cudaError_t e = cudaMemcpyAsync(chi2.data(), h->S.chi2, chi2.size() * 8, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) h->chi2_ref = mean_residue(chi2.data(), h->prm.n_walkers);
+    return e;
+}
+
 // Whether a handle's blocks may run in the span of the kernel's columns at all: own bins, FP32
 // decisions, and neither the loop over tau nor its lanes (the order of its sums) asked for.
 bool span_allowed(const sail_params &p) {
@@ -307,9 +336,11 @@ bool span_allowed(const sail_params &p) {
 // run gives the same result either way, the span sweep takes the blocks in which such a decision
 // is not expected: moves x 1e-7 x S / T of them, 1e-7 the rounding of delta chi2 (and its drift
 // between two recomputations) relative to the magnitude of its terms, S = eps_max |R| (|R| + |Fhat|)
-// that magnitude.  Measured on the paper-scale problem, walkers of 4096 that parted in a block of
-// 4.1e8 moves: 0 at T = 10 chi2_0 .. 0.5 chi2_0 (estimate 0.004 .. 0.06), 7 to 17 at T = 1e6 near
-// equilibrium (estimate 16).  The line lies at 1/64 of a decision a block: at 1/16, 3 of 6 runs of the band
+// that magnitude.  Moves and residue are the whole population's, also on a shard, and the residue is
+// that of the walkers' stored chi2: a shard, the whole population and a restored handle choose alike.
+// Measured on the paper-scale problem, walkers of 4096 that parted in a block of 4.1e8 moves: 0 at
+// T = 10 chi2_0 .. 0.5 chi2_0 (estimate 0.004 .. 0.06), 7 to 17 at T = 1e6 near equilibrium
+// (estimate 16).  The line lies at 1/64 of a decision a block: at 1/16, 3 of 6 runs of the band
 // example (estimate 0.016 a block) parted from the sweep over tau within 6 blocks and 1 of 60 tiny inversions.
 bool span_next(const sail_ctx *h, int n0, int n1) {
     const sail_params &p = h->prm;
@@ -317,7 +348,7 @@ bool span_next(const sail_ctx *h, int n0, int n1) {
     const double T = std::min(h->T[n0], h->T[n1 - 1]);
     const double eps = p.move_scale > 0.0 ? p.move_scale : 1.0 / h->n_omega;
     const double R = std::sqrt(h->chi2_ref), S = eps * R * (R + h->F_norm);
-    const double moves = (double)(n1 - n0) * p.n_walkers * h->n_omega;
+    const double moves = (double)(n1 - n0) * population(h) * h->n_omega;
     return moves * 1e-7 * std::min(1.0, S / T) <= 0.015625;     // chi2 not known (NaN): S / T counts as 1
 }
 
@@ -637,7 +668,7 @@ int sail_create(sail_t *out, const double *tau, const double *F, const double *s
     h->B = B;
     h->lambda0 = lambda;
     h->chi2_0 = chi2_0;
-    h->chi2_ref = chi2_0;
+    h->chi2_ref = mean_residue(std::vector<double>(population(h), chi2_0).data(), population(h));
     h->F_norm = 0.0;
     for (int i = 0; i < n_tau; ++i) h->F_norm += F64[i] * F64[i];
     h->F_norm = std::sqrt(h->F_norm);
@@ -1044,7 +1075,7 @@ int block_finish(sail_ctx *h, const BlockPending &b, sail_block_stats *out) {
         const double proposed = (double)(b.block_end - b.n_begin) * p.n_walkers * h->n_omega;
         h->pos_frac_last = (double)(b.bc.pos - h->pos_seen) / proposed;
     }
-    h->chi2_ref = b.bc.chi2_sum / p.n_walkers;
+    h->chi2_ref = population(h) > p.n_walkers ? NAN : b.bc.chi2_sum / p.n_walkers;
     h->acc_seen = b.bc.acc;
     h->pos_seen = b.bc.pos;
     h->blocks_done += 1;
@@ -1078,6 +1109,7 @@ int sail_anneal(sail_t h, int max_blocks, sail_block_stats *stats, int *n_done) 
         BlockPending b{};
         b.n_begin = h->sweeps_done;
         b.block_end = block_end_of(h);
+        SAIL_CUDA(ref_update(h), "chi2 D2H");
         h->P.span_on = span_next(h, b.n_begin, b.block_end);
         for (int n = b.n_begin; n < b.block_end;) {
             const int next = next_resync(h, n, b.block_end);
@@ -1350,6 +1382,16 @@ int sail_imprint_rows(sail_t h, int n, const int *idx, const double *d_a_rows, c
               "imprint launch");
     h->launches += 1;
     SAIL_CUDA(cudaStreamSynchronize(h->stream), "imprint sync");
+    h->chi2_ref = NAN;
+    return SAIL_OK;
+}
+
+int sail_population_residue(sail_t h, int n_total, const double *chi2_all, double *mean) {
+    if (!h || !chi2_all) return fail(SAIL_EINVAL, "NULL argument");
+    if (n_total != population(h)) return fail(SAIL_EINVAL, "n_total must be %d, the walkers of the population", population(h));
+    const double m = mean_residue(chi2_all, n_total);
+    if (n_total > h->prm.n_walkers) h->chi2_ref = m;      // a whole population's handle knows its own
+    if (mean) *mean = m;
     return SAIL_OK;
 }
 
@@ -1396,17 +1438,10 @@ int sail_restore(sail_t h, const void *buf, size_t bytes) {
     in += (size_t)h->prm.n_sweeps * 8;
     for (const CkptRegion &r : ckpt_regions(h)) {
         SAIL_CUDA(cudaMemcpyAsync(h->ws + r.off, in, r.bytes, cudaMemcpyHostToDevice, h->stream), "restore H2D");
-        if (r.off == h->L.chi2) {
-            double sum = 0.0, c2;
-            for (int w = 0; w < h->prm.n_walkers; ++w) {
-                std::memcpy(&c2, in + (size_t)w * 8, 8);
-                sum += c2;
-            }
-            h->chi2_ref = sum / h->prm.n_walkers;
-        }
         in += r.bytes;
     }
     SAIL_CUDA(cudaStreamSynchronize(h->stream), "restore sync");
+    h->chi2_ref = NAN;
     h->sweeps_done = c.sweeps_done;
     h->blocks_done = c.blocks_done;
     h->events = c.events;
@@ -1731,6 +1766,7 @@ int batch_run_blocks(sail_batch_ctx *b, int max_blocks, int *n_done) {
             pend[k] = BlockPending{};
             pend[k].n_begin = b->h[k]->sweeps_done;
             pend[k].block_end = block_end_of(b->h[k]);
+            SAIL_CUDA(ref_update(b->h[k]), "chi2 D2H");
             b->h[k]->P.span_on = span_next(b->h[k], pend[k].n_begin, pend[k].block_end);
             cur[k] = pend[k].n_begin;
         }

@@ -3,7 +3,9 @@
 Between branching events the walkers are independent (Sec. 2.2), so each shard anneals its own
 contiguous range of the population; its random counters carry the walkers' population indices
 (sail_params.walker_offset), so a shard draws exactly what the whole population would for
-those walkers.  At every block end (Sec. 2.5):
+those walkers.  Before every block each shard is told the whole population's chi2
+(sail_population_residue), by which it chooses the block's sweep as the whole population would.  At
+every block end (Sec. 2.5):
 
   1. every shard's chi2 after the block's residual recomputation is gathered by every process;
   2. every process runs the same deterministic branching solve on the whole population's chi2
@@ -13,13 +15,16 @@ those walkers.  At every block end (Sec. 2.5):
   4. each shard imprints its receivers from those rows (sail_imprint_rows).
 
 The result is the single-handle run's, bit for bit: the same draws, the same solve input, the
-same imprint arithmetic.  This module only orders the steps and moves bytes; the arithmetic runs
+same imprint arithmetic, the same sweep.  (One choice is a shard's own: with sweep_loop = 0 on a
+uniform grid of up to 256 tau points, where the single handle has 16 walkers a SM or more, its blocks
+over tau may look ahead where a smaller shard moves one at a time; the two round delta chi2
+differently in the last bits.  Given sweep_loop = 1 or 2 there is nothing to choose.)  This module only orders the steps and moves bytes; the arithmetic runs
 in the library's kernels.  The geometric schedule is supported; the self-cooling schedule,
 adaptive branching and smoothing need population statistics per block and are not.
 
 Engines (duck-typed): offset, n_walkers, run_block(), chi2() -> float64 array,
 rows(idx) -> (a_rows, R_rows), imprint(idx, a_rows, R_rows, t), solve(chi2_all, block, fraction)
--> (m, Delta, receivers, donors).  CudaShard is the library's; any object with these methods
+-> (m, Delta, receivers, donors), and, if its sweep depends on it, population(chi2_all).  CudaShard is the library's; any object with these methods
 (for instance a CPU model of the method) can be sharded the same way.
 Communicators: LocalComm (all shards in one process) and TorchComm (torch.distributed, one or
 more shards per rank; NCCL with CUDA tensors, gloo with CPU tensors).
@@ -95,6 +100,9 @@ class CudaShard:
     def chi2(self) -> np.ndarray:
         return self.handle.chi2()
 
+    def population(self, chi2_all):
+        self.handle.population_residue(chi2_all)
+
     def rows(self, idx):
         return self.handle.walker_rows(idx)
 
@@ -141,10 +149,8 @@ class ShardedAnneal:
         self.blocks = 0
         self.events: List[dict] = []
 
-    def block(self) -> dict:
-        for s in self.shards:
-            s.run_block()
-        # 1. the whole population's chi2, assembled in population order
+    def _chi2_all(self) -> np.ndarray:
+        """The whole population's chi2, assembled in population order."""
         local = np.concatenate([s.chi2() for s in self.shards]) if self.shards else np.zeros(0)
         gathered = self.comm.all_gather(local, self.counts)
         chi2_all = np.empty(self.n_total)
@@ -153,6 +159,17 @@ class ShardedAnneal:
             for o, n in self.layout[r]:
                 chi2_all[o:o + n] = vals[q:q + n]
                 q += n
+        return chi2_all
+
+    def block(self) -> dict:
+        if hasattr(self.shards[0], "population"):
+            before = self._chi2_all()
+            for s in self.shards:
+                s.population(before)
+        for s in self.shards:
+            s.run_block()
+        # 1. the whole population's chi2
+        chi2_all = self._chi2_all()
         # 2. the same solve on every process
         m, delta, zl, dl = self.shards[0].solve(chi2_all, self.blocks, self.fraction)
         # 3. donor rows: local ones read here, remote ones sent by their owners

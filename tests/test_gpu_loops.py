@@ -109,3 +109,26 @@ def test_paper_grid_blocks_over_tau_and_in_the_basis():
     for other in out[1:]:
         for x, y in zip(out[0], other):
             np.testing.assert_array_equal(np.asarray(x), np.asarray(y))
+
+
+@pytest.mark.parametrize("n_omega,kw", [
+    (1001, {}), (1003, {"hastings": True}), (1006, {"index_walk_len": 2}), (1001, {"index_walk_len": 3}),
+    (1007, {"index_walk_len": 7, "walk_uniform": 0.2}), (1000, {"index_walk_len": 1}),
+])
+def test_hot_blocks_count_and_end_as_over_tau(n_omega, kw):
+    """Same spectra, accepted moves and positivity rejections in the basis and over tau, also where the
+    sweep ends inside a batch of draws; the state was set, so its residue is taken from the walkers."""
+    tau = 8.0 * np.arange(40, dtype=np.float64) / 39
+    P = make_problem("hot", tau, n_omega, 20.0, [Peak("lorentz", 2.0, 0.3, 0.6), Peak("lorentz", 5.0, 0.5, 0.4)], 1e-4, 3, 1)
+    out = []
+    for loop in (0, 1):
+        g = sail.Sail(P.tau, P.F, P.sigma, P.omega,
+                      sail.Params(n_walkers=301, n_sweeps=20000, sweeps_per_block=3, branching=False, A=P.A, B=P.B, seed=11,
+                                  resync_kind=sail.RESYNC_FP32, sweep_loop=loop, **kw))
+        g.set_state(g.state()[0])
+        stats = g.anneal(1)[0]
+        assert g.span_info()["blocks"] == 1 - loop
+        out.append((*g.state()[:4], stats["positivity_rejected"], stats["acceptance"]))
+        g.close()
+    for u, v in zip(*out):
+        np.testing.assert_array_equal(np.asarray(u), np.asarray(v))

@@ -138,3 +138,30 @@ def test_layout_must_tile_the_population():
         ShardedAnneal([Dummy(0, 4)], [[(0, 4), (5, 3)]], LocalComm())
     with pytest.raises(ValueError):
         ShardedAnneal([Dummy(0, 5)], [[(0, 4)]], LocalComm())
+
+
+def test_shards_are_told_the_population_before_every_block():
+    """An engine whose sweep depends on the population gets its chi2 before each block, in index order
+    whatever the order of the shards, as the walkers hold it then (after imprinting)."""
+    from paper_1609_07936_gb300.sharded import LocalComm, ShardedAnneal
+    from workloads import tiny_double_lorentz
+
+    class Told(OracleShard):
+        def __init__(self, *args):
+            super().__init__(*args)
+            self.told = []
+
+        def population(self, chi2_all):
+            self.told.append(np.array(chi2_all))
+
+    P = tiny_double_lorentz()
+    spans = [(10, 14), (0, 10)]
+    shards = [Told(P, o, n) for o, n in spans]
+    run = ShardedAnneal(shards, [spans], LocalComm(), 0.25, 0.1)
+    for b in range(BLOCKS):
+        now = np.concatenate([shards[1].chi2(), shards[0].chi2()])
+        run.block()
+        for s in shards:
+            assert len(s.told) == b + 1
+            np.testing.assert_array_equal(s.told[b], now)
+    assert any((ev["m"] == 0).any() for ev in run.events)
