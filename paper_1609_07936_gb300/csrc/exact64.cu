@@ -849,11 +849,13 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
     }
 }
 
+// room for the kernel's static shared memory (its few hundred bytes of reductions) beside the 128 KiB
+constexpr size_t kSolveStatic = 4096;
 template <int PT>
 cudaError_t launch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision, int block_index,
                          double fraction, int event, cudaStream_t st, int *launches) {
     const size_t staged = (size_t)P.n_walkers * sizeof(double);   // <= 128 KiB (16384 walkers)
-    cudaError_t e = cudaFuncSetAttribute(branch_solve_kernel<PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+    const cudaError_t e = allow_smem(branch_solve_kernel<PT>, kSolveStatic);
     if (e != cudaSuccess) return e;
     branch_solve_kernel<PT><<<1, kSolveThreads, staged, st>>>(P, S, B, block_index, fraction, event, precision == 0);
     *launches += 1;
@@ -1205,7 +1207,7 @@ cudaError_t launch_sweep64_c(const DevProblem &P, const DevState &S, int n0, int
     const int blocks = (P.n_walkers + warps - 1) / warps;
     const size_t staged = warps * sweep64_warp_bytes(true, P.n_omega, C);
     if (staged <= (size_t)smem_max) {
-        const cudaError_t e = cudaFuncSetAttribute(sweep_fp64_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+        const cudaError_t e = allow_smem(sweep_fp64_kernel<C, true>);
         if (e != cudaSuccess) return e;
         sweep_fp64_kernel<C, true><<<blocks, 32 * warps, staged, st>>>(P, S, n0, n1);
     } else {

@@ -104,6 +104,25 @@ struct BranchScratch {
     double *delta_trace;   // [max_events] or null
 };
 
+// Lets every launch of a kernel ask for as much shared memory as a block may have (fixed: bytes the kernel
+// holds besides).  The attribute belongs to the process: every caller sets the same value, so that a
+// launch in another thread cannot lower it between a caller's attribute call and its launch.
+template <typename Kernel>
+cudaError_t allow_smem(Kernel kernel, size_t fixed = 0) {
+    int dev = 0, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)fixed);
+}
+// Static shared memory of a kernel.
+template <typename Kernel>
+cudaError_t static_smem(Kernel kernel, size_t *bytes) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    *bytes = e == cudaSuccess ? a.sharedSizeBytes : 0;
+    return e;
+}
+
 struct BlockCounters {     // device-side block statistics, read back once per block
     double chi2_min, chi2_sum;
     unsigned long long acc, pos;

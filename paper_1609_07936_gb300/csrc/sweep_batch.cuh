@@ -82,7 +82,9 @@ cudaError_t launch_batch_g(const BatchProblem *d_probs, const BatchItem *d_items
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     constexpr int kMaxWarps = sweep_threads<G, G == 8 ? 8 : 16>() / 32;
     if (warps > kMaxWarps) warps = kMaxWarps;
-    cudaError_t e = cudaFuncSetAttribute(sweep_batch_kernel<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    size_t fixed = 0;
+    cudaError_t e = static_smem(sweep_batch_kernel<G, MODE>, &fixed);
+    if (e == cudaSuccess) e = allow_smem(sweep_batch_kernel<G, MODE>, fixed);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(d_counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;

@@ -1204,8 +1204,7 @@ cudaError_t launch_c(const DevProblem &P, const DevState &S, int n0, int n1, cud
     if (tb > (size_t)smem_max) return cudaErrorInvalidValue;
     Gm.stage_b = tb + staged <= (size_t)smem_max;
     const size_t smem = tb + (Gm.stage_b ? staged : 0);
-    cudaError_t e = cudaFuncSetAttribute(sweep_fp32_kernel<G, C, MODE, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(sweep_fp32_kernel<G, C, MODE, AHEAD>);
     if (e != cudaSuccess) return e;
     const int n_ctas = (Gm.groups_total + Gm.groups_per_cta - 1) / Gm.groups_per_cta;
     sweep_fp32_kernel<G, C, MODE, AHEAD><<<n_ctas, Gm.warps * 32, smem, st>>>(P, S, n0, n1, Gm);

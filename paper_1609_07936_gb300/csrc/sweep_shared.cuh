@@ -401,8 +401,7 @@ cudaError_t launch_shared_c(const DevProblem &P, const DevState &S, int n0, int 
     if (tb > (size_t)smem_max) return cudaErrorInvalidValue;
     Gm.stage_b = tb + staged <= (size_t)smem_max;
     const size_t smem = tb + (Gm.stage_b ? staged : 0);
-    cudaError_t e = cudaFuncSetAttribute(sweep_shared_kernel<W, C, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(sweep_shared_kernel<W, C, MODE>);
     if (e != cudaSuccess) return e;
     const int n_ctas = (Gm.groups_total + Gm.groups_per_cta - 1) / Gm.groups_per_cta;
     sweep_shared_kernel<W, C, MODE><<<n_ctas, Gm.warps * 32, smem, st>>>(P, S, n0, n1, Gm);

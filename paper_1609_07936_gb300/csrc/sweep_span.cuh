@@ -611,7 +611,7 @@ SpanGeom span_geom(const DevProblem &P, int sms, int smem_max, size_t *smem) {
 template <int RR, int G, int MODE, int LM = 0>
 cudaError_t launch_span_g(const DevProblem &P, const DevState &S, int n0, int n1, const SpanGeom &Gm, size_t smem,
                           cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(sweep_span_kernel<RR, G, MODE, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(sweep_span_kernel<RR, G, MODE, LM>);
     if (e != cudaSuccess) return e;
     const int n_ctas = (Gm.groups_total + Gm.groups_per_cta - 1) / Gm.groups_per_cta;
     sweep_span_kernel<RR, G, MODE, LM><<<n_ctas, Gm.warps * 32, smem, st>>>(P, S, n0, n1, Gm);
@@ -702,16 +702,6 @@ __global__ void __launch_bounds__(32 * kSpanWarps, 1) sweep_span_batch_kernel(co
     }
 }
 
-// Shared memory the kernel holds besides the launch's: the two together must stay within the device's
-// limit per block.
-template <int G, int MODE>
-cudaError_t span_batch_static(size_t *bytes) {
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, sweep_span_batch_kernel<G, MODE>);
-    *bytes = e == cudaSuccess ? a.sharedSizeBytes : 0;
-    return e;
-}
-
 template <int G, int MODE>
 cudaError_t launch_span_batch_g(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
                                 size_t smem, int warps, cudaStream_t st) {
@@ -719,7 +709,9 @@ cudaError_t launch_span_batch_g(const BatchProblem *d_probs, const BatchItem *d_
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (warps > kSpanWarps) warps = kSpanWarps;
-    cudaError_t e = cudaFuncSetAttribute(sweep_span_batch_kernel<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    size_t fixed = 0;
+    cudaError_t e = static_smem(sweep_span_batch_kernel<G, MODE>, &fixed);
+    if (e == cudaSuccess) e = allow_smem(sweep_span_batch_kernel<G, MODE>, fixed);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(d_counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;

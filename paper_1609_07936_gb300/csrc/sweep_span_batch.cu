@@ -14,7 +14,7 @@ cudaError_t span_batch_smem(const DevProblem &P, int mode, size_t *bytes) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     size_t fixed = 0;
-    const cudaError_t e = mode == kPlain ? span_batch_static<4, kPlain>(&fixed) : span_batch_static_modes(mode, &fixed);
+    const cudaError_t e = mode == kPlain ? static_smem(sweep_span_batch_kernel<4, kPlain>, &fixed) : span_batch_static_modes(mode, &fixed);
     if (e != cudaSuccess) return e;
     const size_t base = span_ring_bytes(kSpanWarps) + (size_t)span_vec_floats(P.n_omega) * 4;
     const size_t all = base + (size_t)P.n_omega * P.span * 4;

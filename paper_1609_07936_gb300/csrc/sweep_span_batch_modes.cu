@@ -4,7 +4,7 @@
 namespace sail {
 
 cudaError_t span_batch_static_modes(int mode, size_t *bytes) {
-    return mode == kWalk ? span_batch_static<8, kWalk>(bytes) : span_batch_static<8, kHastings>(bytes);
+    return mode == kWalk ? static_smem(sweep_span_batch_kernel<8, kWalk>, bytes) : static_smem(sweep_span_batch_kernel<8, kHastings>, bytes);
 }
 
 cudaError_t launch_span_batch_modes(const BatchProblem *d_probs, const BatchItem *d_items, int n_items, int *d_counter,
