@@ -1327,7 +1327,7 @@ int sail_branch_solve(sail_t h, int n_total, const double *chi2_all, int block, 
     B.m_trace = nullptr;
     B.delta_trace = nullptr;
     int l = 0;
-    SAIL_CUDA(launch_branch_solve(P, S, B, h->prm.precision, block, fraction, st, &l), "solve launch");
+    SAIL_CUDA(launch_branch_solve(P, S, B, block, fraction, st, &l), "solve launch");
     h->launches += l;
     int np = 0;
     SAIL_CUDA(cudaMemcpyAsync(m, B.m, (size_t)n_total * 4, cudaMemcpyDeviceToHost, st), "solve D2H");

@@ -589,6 +589,112 @@ __device__ int multipliers_at(int N, const double *z, const double *xi, double D
     return block_sum_i(zc, sh);
 }
 
+// The sum of the walkers' residues in walker order, every partial sum rounded as one FP64 addition
+// rounds it, by a whole block.  While the running sum stays in one binade it is an integer S in units
+// of its last place, and adding c adds an integer to S: c in that unit, rounded to nearest, a tie to
+// the even sum.  A step is then what S grows by if it is even and if it is odd; steps compose, so a
+// scan over the walkers gives S at every walker up to the one whose addition leaves the binade, and
+// that addition is done as such.  One thread's chain of additions (some 60 cycles each) took 0.53 ms
+// at 16384 walkers and 0.07 ms at 2000; this takes a scan for every doubling of the sum past its first
+// 64 terms, 0.14 and 0.02 ms.
+struct SumStep { unsigned long long even, odd; };
+constexpr unsigned long long kSumTop = 1ull << 53;      // S leaves the binade
+__host__ __device__ __forceinline__ SumStep sum_then(SumStep a, SumStep b) {
+    // saturated well past the binade, where the parity no longer matters
+    const unsigned long long e = a.even + (a.even & 1 ? b.odd : b.even), o = a.odd + (a.odd & 1 ? b.even : b.odd);
+    return {e < 2 * kSumTop ? e : 2 * kSumTop, o < 2 * kSumTop ? o : 2 * kSumTop};
+}
+// The step of adding c >= 0 (its bits) to a sum whose biased exponent is e.
+__host__ __device__ __forceinline__ SumStep sum_step(unsigned long long c, int e) {
+    const int k = (int)(c >> 52) & 0x7FF;
+    const unsigned long long m = (c & (kSumTop / 2 - 1)) | (k ? kSumTop / 2 : 0);
+    const int low = e - (k ? k : 1);                    // places of c below the sum's last
+    if (low <= 0) {
+        const unsigned long long q = low < -1 ? 2 * kSumTop : m << -low;
+        return {q, q};
+    }
+    if (low > 53) return {0, 0};
+    const unsigned long long q = m >> low, rest = m & ((1ull << low) - 1), half = 1ull << (low - 1);
+    if (rest == half) return {q + (q & 1), q + ((q + 1) & 1)};
+    return {q + (rest > half), q + (rest > half)};
+}
+// Where walker l's residue stands in shared memory: threads that read 16, 8 or 4 consecutive ones meet
+// different banks.
+__host__ __device__ __forceinline__ int sum_at(int l) { return l + (l >> 4); }
+
+struct SumShared {
+    double s;            // the sum of the first `at` residues
+    int at;
+    SumStep warp[32];
+};
+// c: N residues at sum_at(l), stored by all threads before a barrier.  Values that are not residues (NaN,
+// negative, huge) and sums below the normal range are added one by one.
+template <int PT>
+__device__ double ordered_sum(const double *c, int N, SumShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int first = tid * PT;
+    bool plain = true;
+    for (int l = first; l < min(N, first + PT); ++l) plain = plain && c[sum_at(l)] >= 0.0 && c[sum_at(l)] <= 1e300;
+    const bool scan = __syncthreads_and(plain);
+    if (tid == 0) {
+        double s = 0.0;
+        const int n = scan ? min(N, 64) : N;
+        for (int l = 0; l < n; ++l) s += c[sum_at(l)];
+        if (!(s >= 1e-290))
+            for (int l = n; l < N; ++l) s += c[sum_at(l)];
+        sh.s = s;
+        sh.at = s >= 1e-290 ? n : N;
+    }
+    for (;;) {
+        __syncthreads();
+        const double s = sh.s;
+        const int at = sh.at;
+        if (at >= N) return s;
+        const unsigned long long bits = __double_as_longlong(s);
+        const int e = (int)(bits >> 52);
+        const unsigned long long S = (bits & (kSumTop / 2 - 1)) | kSumTop / 2;
+        SumStep own = {0, 0};
+        for (int l = max(at, first); l < min(N, first + PT); ++l) own = sum_then(own, sum_step(__double_as_longlong(c[sum_at(l)]), e));
+        SumStep incl = own;
+        auto up = [&](SumStep v, int o) -> SumStep { return {__shfl_up_sync(kFull, v.even, o), __shfl_up_sync(kFull, v.odd, o)}; };
+        for (int o = 1; o < 32; o <<= 1) {
+            const SumStep t = up(incl, o);
+            if (lane >= o) incl = sum_then(t, incl);
+        }
+        if (lane == 31) sh.warp[warp] = incl;
+        SumStep before = up(incl, 1);
+        if (lane == 0) before = {0, 0};
+        __syncthreads();
+        SumStep w = sh.warp[lane];                      // 32 warps
+        for (int o = 1; o < 32; o <<= 1) {
+            const SumStep t = up(w, o);
+            if (lane >= o) w = sum_then(t, w);
+        }
+        const SumStep all = {__shfl_sync(kFull, w.even, 31), __shfl_sync(kFull, w.odd, 31)};
+        const SumStep off = {__shfl_sync(kFull, w.even, (warp + 31) & 31), __shfl_sync(kFull, w.odd, (warp + 31) & 31)};
+        if (warp > 0) before = sum_then(off, before);
+        const SumStep after = sum_then(before, own);
+        auto at_S = [S](SumStep v) { return S + (S & 1 ? v.odd : v.even); };
+        auto value = [e](unsigned long long v) { return __longlong_as_double(((unsigned long long)e << 52) | (v & (kSumTop / 2 - 1))); };
+        if (at_S(before) < kSumTop && at_S(after) >= kSumTop) {
+            unsigned long long v = at_S(before);
+            for (int l = max(at, first); l < N; ++l) {
+                const SumStep step = sum_step(__double_as_longlong(c[sum_at(l)]), e);
+                const unsigned long long next = v + (v & 1 ? step.odd : step.even);
+                if (next >= kSumTop) {
+                    sh.s = value(v) + c[sum_at(l)];
+                    sh.at = l + 1;
+                    break;
+                }
+                v = next;
+            }
+        } else if (tid == 0 && at_S(all) < kSumTop) {
+            sh.s = value(at_S(all));
+            sh.at = N;
+        }
+    }
+}
+
 // The whole solve in one block: the search over Delta is sequential, and a trial is cheap because
 // FP32 decides nearly every multiplier.  At a trial Delta each thread holds e^(-Delta z_l) in FP32
 // with a bound on its error; a count of sum m at some Theta forms Theta E + xi in FP32 and goes to
@@ -677,10 +783,11 @@ struct SolveSearch {
 
 template <int PT>
 __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProblem P, DevState S, BranchScratch B, int block_index,
-                                                                        double fraction, int event, int ordered) {
-    extern __shared__ double s_chi2[];           // chi2 [N] for the ordered sum; then z [N] and the draws [N]
+                                                                        double fraction, int event) {
+    extern __shared__ double s_chi2[];           // chi2 for the ordered sum; then z [N] and the draws [N]
     __shared__ SolveShared sh;
     __shared__ SolveSearch s_search;
+    __shared__ SumShared s_sum;
     __shared__ int2 red[2][32];
     __shared__ float red_f[2][32];
     const int N = P.n_walkers, tid = threadIdx.x;
@@ -688,11 +795,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
     uint32_t *s_word = reinterpret_cast<uint32_t *>(s_z + N);
     int Zt = (int)floor(fraction * N + 0.5);
     if (Zt > N - 1) Zt = N - 1;
-    double cmin = S.chi2[0], part = 0.0;
+    double cmin = S.chi2[0];
     for (int l = tid; l < N; l += kSolveThreads) {
         const double c = S.chi2[l];
-        if (ordered) s_chi2[l] = c;
-        else part += c;
+        s_chi2[sum_at(l)] = c;
         cmin = c < cmin ? c : cmin;
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -706,20 +812,8 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
         const double c = __shfl_xor_sync(kFull, cmin, o);
         cmin = c < cmin ? c : cmin;
     }
-    // the mean: FP64 state sums in walker order (the validation path's), FP32 state over threads
-    double csum;
-    if (ordered) {
-        if (tid == 0) {
-            double c = 0.0;
-#pragma unroll 8
-            for (int l = 0; l < N; ++l) c += s_chi2[l];
-            sh.theta = c;
-        }
-        __syncthreads();
-        csum = sh.theta;
-    } else {
-        csum = block_sum_d(part, sh);
-    }
+    // the mean, summed in the oracle's order: where the residues lie close together, z hangs on its last bits
+    const double csum = ordered_sum<PT>(s_chi2, N, s_sum);
     const double spread = csum / N - cmin;
     const float scale = spread > 0.0 ? (float)(1.0 / spread) : 0.0f;
     const uint2 key = philox_key(P.seed);
@@ -849,15 +943,15 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
     }
 }
 
-// room for the kernel's static shared memory (its few hundred bytes of reductions) beside the 128 KiB
+// room for the kernel's static shared memory (its reductions, under 2 KiB) beside the 136 KiB
 constexpr size_t kSolveStatic = 4096;
 template <int PT>
-cudaError_t launch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision, int block_index,
-                         double fraction, int event, cudaStream_t st, int *launches) {
-    const size_t staged = (size_t)P.n_walkers * sizeof(double);   // <= 128 KiB (16384 walkers)
+cudaError_t launch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int block_index, double fraction,
+                         int event, cudaStream_t st, int *launches) {
+    const size_t staged = (size_t)(sum_at(P.n_walkers - 1) + 1) * sizeof(double);   // <= 136 KiB (16384 walkers)
     const cudaError_t e = allow_smem(branch_solve_kernel<PT>, kSolveStatic);
     if (e != cudaSuccess) return e;
-    branch_solve_kernel<PT><<<1, kSolveThreads, staged, st>>>(P, S, B, block_index, fraction, event, precision == 0);
+    branch_solve_kernel<PT><<<1, kSolveThreads, staged, st>>>(P, S, B, block_index, fraction, event);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -1404,16 +1498,16 @@ cudaError_t launch_resync(const DevProblem &P, const DevState &S, int precision,
 cudaError_t launch_branch(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision,
                           int block_index, double fraction, double imprint_t, int event, cudaStream_t st,
                           int *launches) {
-    const cudaError_t e = launch_solve_n(P, S, B, precision, block_index, fraction, event, st, launches);
+    const cudaError_t e = launch_solve_n(P, S, B, block_index, fraction, event, st, launches);
     if (e != cudaSuccess) return e;
     imprint_kernel<<<P.n_walkers, 128, 0, st>>>(P, S, B, precision, imprint_t);
     *launches += 1;
     return cudaGetLastError();
 }
 
-cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision,
-                                int block_index, double fraction, cudaStream_t st, int *launches) {
-    return launch_solve_n(P, S, B, precision, block_index, fraction, 0, st, launches);
+cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int block_index,
+                                double fraction, cudaStream_t st, int *launches) {
+    return launch_solve_n(P, S, B, block_index, fraction, 0, st, launches);
 }
 
 cudaError_t launch_walker_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,

@@ -185,8 +185,8 @@ cudaError_t launch_branch(const DevProblem &P, const DevState &S, const BranchSc
                           int event, cudaStream_t st, int *launches);
 // The branching solve alone (multipliers, Delta, imprint pairs into B) over P.n_walkers chi2
 // values in S.chi2, draws keyed by population index (P.walker_base + l); no imprint, no trace.
-cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int precision,
-                                int block_index, double fraction, cudaStream_t st, int *launches);
+cudaError_t launch_branch_solve(const DevProblem &P, const DevState &S, const BranchScratch &B, int block_index,
+                                double fraction, cudaStream_t st, int *launches);
 // Rows of walkers idx[0..n) (device array) in FP64, and imprinting of walkers idx from donor rows.
 cudaError_t launch_walker_rows(const DevProblem &P, const DevState &S, int precision, int n, const int *idx,
                                double *a_rows, double *R_rows, cudaStream_t st);

@@ -45,3 +45,29 @@ def test_solve_gives_the_oracle_multipliers(n, kind, precision):
         np.testing.assert_array_equal(donor, np.repeat(np.arange(n), np.maximum(m - 1, 0))[: zero.size])
         assert zero.size == (m == 0).sum()
     g.close()
+
+
+@pytest.mark.parametrize("precision", [sail.PREC_FP64, sail.PREC_FP32])
+@pytest.mark.parametrize("n", [2, 33, 64, 65, 1024, 1025, 4097, 8193, 16384])
+def test_solve_of_a_population_with_close_residues(n, precision):
+    """Residues within 1e-10 of each other and less: z = (chi2 - min) / (mean - min) hangs on the mean's last
+    bits, so the solve is the oracle's only if its sum is rounded like the oracle's, one walker after
+    the other; also where most additions are ties (residues on a grid of 2^-13 near 2^40), and where
+    the sum passes many binades, ends in the first, or holds zeros."""
+    P = tiny_double_lorentz()
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega,
+                  sail.Params(n_walkers=2, precision=precision, n_sweeps=10, branching=False, A=P.A, B=P.B, seed=5,
+                              walker_total=16384))
+    rng = np.random.default_rng(n)
+    ramp = np.sort(np.exp(12.0 * rng.standard_normal(n)))
+    huge = np.zeros(n)
+    huge[0] = 1e6
+    cases = [_chi2("near", n, 1e-10), _chi2("near", n, 1e-12), _chi2("near", n, 1e-14),
+             2.0**40 + rng.integers(0, 200, n) / 8192.0, ramp, ramp[::-1], huge, np.where(rng.random(n) < 0.5, 0.0, 3.0)]
+    for c in cases:
+        for block in range(3):
+            m, delta, _, _ = g.branch_solve(c, block, 0.25)
+            m_o, delta_o = O.branch_multipliers(c, O.xi_for_block(5, block, n), 0.25)[:2]
+            assert delta == delta_o
+            np.testing.assert_array_equal(m, m_o)
+    g.close()
