@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
     // the mean, summed in the oracle's order: where the residues lie close together, z hangs on its last bits
     const double csum = ordered_sum<PT>(s_chi2, N, s_sum);
     const double spread = csum / N - cmin;
-    const float scale = spread > 0.0 ? (float)(1.0 / spread) : 0.0f;
+    const double scale = spread > 0.0 ? 1.0 / spread : 0.0;    // FP64: residues and mean may leave FP32's range, z does not
     const uint2 key = philox_key(P.seed);
     __syncthreads();
     float xif[PT], E[PT];                        // this thread's walkers: draws, and E at the trial Delta
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
         m[q] = 1;
         if (l < N) {
             const uint32_t w = philox4x32_10(make_uint4((uint32_t)(l + P.walker_base), (uint32_t)block_index, 0u, 1u), key).x;
-            s_z[l] = scale * (float)(S.chi2[l] - cmin);
+            s_z[l] = (float)(scale * (S.chi2[l] - cmin));
             s_word[l] = w;
             xif[q] = fmaf((float)w, 2.3283064e-10f, 1.1641532e-10f);
         }

@@ -71,3 +71,26 @@ def test_solve_of_a_population_with_close_residues(n, precision):
             assert delta == delta_o
             np.testing.assert_array_equal(m, m_o)
     g.close()
+
+
+@pytest.mark.parametrize("precision", [sail.PREC_FP64, sail.PREC_FP32])
+@pytest.mark.parametrize("scale", [1e-300, 1e-60, 1e-48, 1e-44, 1e-41, 1e-38, 1e30, 1e35, 1e37, 1e38, 1e39, 1e41, 1e44, 1e47, 1e60, 1e290, 1e296])
+def test_solve_at_any_scale_of_the_residues(scale, precision):
+    """The multipliers depend on the residues' ratios alone: residues whose differences, mean or its inverse
+    leave FP32's range, at either end, give the oracle's; also where one walker lies far above all the
+    others, whose z is then small and Delta large."""
+    P = tiny_double_lorentz()
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega,
+                  sail.Params(n_walkers=2, precision=precision, n_sweeps=10, branching=False, A=P.A, B=P.B, seed=5,
+                              walker_total=16384))
+    for n in (33, 1025, 4097):
+        x = np.random.default_rng(n).standard_normal(n)
+        far = np.exp(0.3 * x)
+        far[n // 2] = 1e8
+        for c in (np.exp(0.3 * x), np.exp(5.0 * np.minimum(x, 2.0)), 1.0 + 1e-3 * np.abs(x), far):
+            for block in range(2):
+                m, delta, _, _ = g.branch_solve(scale * c, block, 0.25)
+                m_o, delta_o = O.branch_multipliers(scale * c, O.xi_for_block(5, block, n), 0.25)[:2]
+                assert delta == delta_o
+                np.testing.assert_array_equal(m, m_o)
+    g.close()
