@@ -204,7 +204,7 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
 // 1 - eps over one launch): one Newton step y + y (1 - g y) in fused arithmetic from the hardware's
 // approximation (Markstein, "Computation of elementary functions on the IBM RISC System/6000
 // processor", 1990).  Equal to 1.0f / g for all 2^23 significands at every exponent from 2^-125 to
-// 2^125 (checked on the GPU).
+// 2^125 and either sign (tests/test_gpu_reciprocal.py).
 __device__ __forceinline__ float rcp_rn(float g) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(g));
