@@ -1226,7 +1226,8 @@ int sail_get_trace(sail_t h, int *acc, int *m, double *delta, int *n_events) {
 namespace {
 
 // Checkpoint layout: a header, the host-side schedule state, then device regions in a fixed
-// order (each region's bytes as the workspace holds them).
+// order (each region's bytes as the workspace holds them), then the positivity-rejected share of the
+// last block, which the automatic move loop follows (buffers of before it was kept end without it).
 struct CkptHeader {
     char magic[8];
     int version, n_tau, n_omega, n_walkers, precision, n_sweeps, sweeps_per_block, resync_every, trace;
@@ -1237,6 +1238,8 @@ struct CkptHeader {
     unsigned long long acc_seen, pos_seen, acc_before;
     double acc_ref, T_freeze, chi2_of_mean;
 };
+
+constexpr size_t kCkptTail = sizeof(double);
 
 struct CkptRegion {
     size_t off, bytes;
@@ -1272,7 +1275,7 @@ std::vector<CkptRegion> ckpt_regions(const sail_ctx *h) {
 size_t ckpt_bytes(const sail_ctx *h) {
     size_t n = sizeof(CkptHeader) + (size_t)h->prm.n_sweeps * 8;   // header and the host T table
     for (const CkptRegion &r : ckpt_regions(h)) n += r.bytes;
-    return n;
+    return n + kCkptTail;
 }
 
 CkptHeader ckpt_header(const sail_ctx *h) {
@@ -1415,6 +1418,7 @@ int sail_checkpoint(sail_t h, void *buf, size_t bytes) {
         out += r.bytes;
     }
     SAIL_CUDA(cudaStreamSynchronize(h->stream), "checkpoint sync");
+    std::memcpy(out, &h->pos_frac_last, kCkptTail);
     return SAIL_OK;
 }
 
@@ -1430,7 +1434,8 @@ int sail_restore(sail_t h, const void *buf, size_t bytes) {
         c.resync_every != mine.resync_every || c.trace != mine.trace || c.schedule_kind != mine.schedule_kind ||
         c.branching != mine.branching || c.seed != mine.seed)
         return fail(SAIL_EINVAL, "checkpoint of a different problem or schedule");
-    if (bytes < ckpt_bytes(h)) return fail(SAIL_EINVAL, "checkpoint has %zu bytes, needs %zu", bytes, ckpt_bytes(h));
+    const size_t need = ckpt_bytes(h) - kCkptTail;
+    if (bytes < need) return fail(SAIL_EINVAL, "checkpoint has %zu bytes, needs %zu", bytes, need);
     if (c.sweeps_done < 0 || c.sweeps_done > c.n_sweeps || c.events < 0 || c.events > h->L.max_events)
         return fail(SAIL_EINVAL, "checkpoint position out of range");
     const char *in = (const char *)buf + sizeof c;
@@ -1442,6 +1447,9 @@ int sail_restore(sail_t h, const void *buf, size_t bytes) {
     }
     SAIL_CUDA(cudaStreamSynchronize(h->stream), "restore sync");
     h->chi2_ref = NAN;
+    h->pos_frac_last = -1.0;
+    if (h->ahead_auto) h->P.ahead = 1;          // the create-time choice, until a block's rejections are known
+    if (bytes >= need + kCkptTail) std::memcpy(&h->pos_frac_last, in, kCkptTail);
     h->sweeps_done = c.sweeps_done;
     h->blocks_done = c.blocks_done;
     h->events = c.events;

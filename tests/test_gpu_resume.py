@@ -73,3 +73,32 @@ def test_restore_refuses_another_problem():
         g.restore(blob[:100])
     g.close()
     h.close()
+
+
+def test_resumed_run_keeps_the_automatic_move_loop():
+    """The automatic loop follows the last block's rejections, which a resumed run knows: 16 walkers a SM
+    on the to-target schedule (about 25% rejections) move one at a time after the first block, as
+    the uninterrupted run does.  A buffer without that share (of an earlier library) is still taken."""
+    import torch
+    W = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    P = paper_scale_double_lorentz(1e-4, n_walkers=W)
+    prm = sail.Params(n_walkers=W, n_sweeps=20000, sweeps_per_block=20, resync_every=10, T_start_abs=1e6, T_end_abs=0.03,
+                      move_scale=0.1 / P.n_omega, A=P.A, B=P.B, seed=8, resync_kind=sail.RESYNC_TENSOR_BF16)
+    g = sail.Sail(P.tau, P.F, P.sigma, P.omega, prm)
+    stats = g.anneal(2)
+    assert stats[-1]["positivity_rejected"] < 0.30 and g.info()["sweep_ahead"] == 0
+    blob = g.checkpoint()
+    h = sail.Sail(P.tau, P.F, P.sigma, P.omega, prm)
+    assert h.info()["sweep_ahead"] == 1
+    h.restore(blob)
+    assert h.info()["sweep_ahead"] == 0
+    for s in (g, h):
+        s.anneal(2)
+    for x, y in zip(g.state()[:4], h.state()[:4]):
+        np.testing.assert_array_equal(x, y)
+    h.restore(blob[:-8])
+    assert h.info()["sweeps_done"] == 40 and h.info()["sweep_ahead"] == 1
+    with pytest.raises(sail.SailError):
+        h.restore(blob[:-9])
+    g.close()
+    h.close()
