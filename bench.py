@@ -182,6 +182,49 @@ def kernel_traffic():
         return None
 
 
+def sweep_roofline(kind, blocks, width, args, smem_gbs, fp32_peak, sms, sm_max_mhz):
+    """Roofline fields of the timed blocks of one kind ("tau": the loops over tau, "span": the sweep in
+    the basis of the kernel's columns); blocks: (moves, sweep ms, launches, statistics) each."""
+    moves, ms, launches = (sum(b[q] for b in blocks) for q in range(3))
+    pos = sum(b[3]["positivity_rejected"] for b in blocks) / len(blocks)
+    acc = sum(b[3]["acceptance"] for b in blocks) / len(blocks)
+    # algorithmic bytes of a walker-move (Sec. 2.2: the update needs the two kernel columns of
+    # the proposed bins and nothing else of their size): b_p and b_s read and, on acceptance,
+    # written (16 B); then, unless the move fails the positivity test (checked before delta
+    # chi2), the columns of p and s in FP32 (N_tau elements each, or the basis's directions)
+    terms = width if kind == "span" else N_TAU
+    bytes_per_move = 16 + (1.0 - pos) * 2 * terms * 4
+    rule = f"16 + (1 - positivity-rejected fraction {pos:.4f}) x 2 x {terms} x 4"
+    if args.shared_bins:
+        # shared bins: a group of W walkers reads one move's columns once
+        bytes_per_move = 16 + 2 * terms * 4 / args.shared_bins
+        rule = f"16 + 2 x {terms} x 4 / {args.shared_bins} (columns read once per group of {args.shared_bins} walkers)"
+    # the sweep is bound by FP32 arithmetic issue and its latency (not HBM, no contraction):
+    # algorithmic FP32 work of a walker-move (Sec. 2.2), per element: for a move that passes
+    # the positivity test d_i = eps M_i - delta_p K_ip - delta_s K_is (1 multiply + 2 FMA =
+    # 5 flops) and d_i (2 R_i + d_i) accumulated (2 FMA = 4 flops); for an accepted move
+    # R_i += d_i, M_i -= d_i (2 flops).  Peak: SMs x 128 FP32 lanes x 2 flops (FMA) x the
+    # maximum SM clock.
+    flops_per_move = terms * (9.0 * (1.0 - pos) + 2.0 * acc)
+    per_launch = moves / max(launches, 1)
+    launch_ms = ms / max(launches, 1)
+    achieved = per_launch * bytes_per_move / (launch_ms * 1e-3) / 1e9
+    flops = per_launch * flops_per_move / (launch_ms * 1e-3) / 1e12
+    kernel = "sweep_span" if kind == "span" else "sweep_shared" if args.shared_bins else "sweep_fp32"
+    return {"kernel": kernel, "bound": "smem", "achieved": achieved, "peak": smem_gbs, "unit": "GB/s", "frac": achieved / smem_gbs,
+            "traffic": kernel_traffic() if kernel == "sweep_fp32" and not args.index_walk else None,
+            "traffic_note": "DRAM bytes per sweep launch (ncu); the sweep's operands live in shared memory",
+            "blocks": len(blocks), "sweep_ms": ms, "moves_per_s": moves / (ms * 1e-3),
+            "algorithmic_bytes_per_move": bytes_per_move, "bytes_per_move_rule": rule,
+            "moves_per_launch": per_launch, "launch_ms": launch_ms,
+            "achieved_rule": "moves_per_launch x algorithmic_bytes_per_move / launch_ms (CUDA events around "
+                             "every sweep launch of these blocks on the handle's stream)",
+            "alu": {"bound": "alu", "achieved": flops, "peak": fp32_peak, "unit": "TFLOP/s", "frac": flops / fp32_peak,
+                    "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {sm_max_mhz:.0f} MHz",
+                    "algorithmic_flops_per_move": flops_per_move,
+                    "flops_per_move_rule": f"{terms} x (9 x (1 - positivity-rejected {pos:.4f}) + 2 x accepted {acc:.4f})"}}
+
+
 def run_gpu(args, rank, world, local_rank):
     import torch
     import paper_1609_07936_gb300 as sail
@@ -227,9 +270,10 @@ def run_gpu(args, rank, world, local_rank):
         time.sleep(0.3)
         barrier()
         e0.record(st)
-        stats = []
+        stats, marks = [], [(info0, 0)]
         for k in range(args.steps):
             stats += g.anneal(1)
+            marks.append((g.info(), g.span_info()["blocks"]))
             flush.zero_()       # L2 flushed between steps (256 MiB write on the same stream)
         e1.record(st)
         barrier()
@@ -237,38 +281,21 @@ def run_gpu(args, rank, world, local_rank):
     info1 = g.info()
     ms_max, moves, value = aggregate(ms, info1["moves"] - info0["moves"], dist, "cuda")
     sweep_ms = info1["sweep_ms"] - info0["sweep_ms"]
-    sweep_n = info1["sweep_launches"] - info0["sweep_launches"]
     launches = info1["kernel_launches"] - info0["kernel_launches"] + args.steps  # + one flush per step
     own_launches = info1["kernel_launches"] - info0["kernel_launches"]
-    moves_per_launch = (info1["moves"] - info0["moves"]) / max(sweep_n, 1)
-    # algorithmic bytes of a walker-move (Sec. 2.2: the update needs the two kernel columns of
-    # the proposed bins and nothing else of size N_tau): b_p and b_s read and, on acceptance,
-    # written (16 B); then, unless the move fails the positivity test (checked before delta
-    # chi2), the columns Khat_p and Khat_s in FP32 (2 N_tau 4 B)
-    col_bytes = 2 * N_TAU * 4
-    pos_frac = sum(b["positivity_rejected"] for b in stats) / max(len(stats), 1)
-    bytes_per_move = 16 + (1.0 - pos_frac) * col_bytes
-    bytes_rule = f"16 + (1 - positivity-rejected fraction {pos_frac:.4f}) x 2 x {N_TAU} x 4"
-    if args.shared_bins:
-        # shared bins: a group of W walkers reads one move's columns once
-        bytes_per_move = 16 + col_bytes / args.shared_bins
-        bytes_rule = f"16 + 2 x {N_TAU} x 4 / {args.shared_bins} (columns read once per group of {args.shared_bins} walkers)"
-
-    launch_s = sweep_ms / max(sweep_n, 1) * 1e-3
-    achieved = moves_per_launch * bytes_per_move / launch_s / 1e9
     clk = clocks.summary(local_rank)
-    # the sweep is bound by FP32 arithmetic issue and its latency (not HBM, no contraction):
-    # algorithmic FP32 work of a walker-move (Sec. 2.2), per tau point: for a move that passes
-    # the positivity test d_i = eps M_i - delta_p Khat_ip - delta_s Khat_is (1 multiply + 2 FMA =
-    # 5 flops) and d_i (2 R_i + d_i) accumulated (2 FMA = 4 flops); for an accepted move
-    # R_i += d_i, M_i -= d_i (2 flops).  Peak: SMs x 128 FP32 lanes x 2 flops (FMA) x the
-    # maximum SM clock.
-    acc_frac = sum(b["acceptance"] for b in stats) / max(len(stats), 1)
-    flops_per_move = N_TAU * (9.0 * (1.0 - pos_frac) + 2.0 * acc_frac)
     sms = torch.cuda.get_device_properties(local_rank).multi_processor_count
     sm_max_mhz = clk.get("sm_max_mhz") or 2070.0
     fp32_peak = sms * 128 * 2 * sm_max_mhz * 1e6 / 1e12
-    fp32_achieved = moves_per_launch * flops_per_move / launch_s / 1e12
+    # blocks swept over tau and blocks swept in the basis of the kernel's columns, apart: they run
+    # different kernels with different work per move
+    width = g.span_info()["width"]
+    part = {"tau": [], "span": []}
+    for (a, na), (b, nb), stat in zip(marks[:-1], marks[1:], stats):
+        part["span" if nb > na else "tau"].append((b["moves"] - a["moves"], b["sweep_ms"] - a["sweep_ms"],
+                                                   b["sweep_launches"] - a["sweep_launches"], stat))
+    rooflines = {k: sweep_roofline(k, v, width, args, smem_gbs, fp32_peak, sms, sm_max_mhz) for k, v in part.items() if v}
+    longest = max(rooflines, key=lambda k: rooflines[k]["sweep_ms"])
 
     # end to end through the public API from host buffers: create (H2D of inputs and tables),
     # K blocks (per-block statistics D2H), average (D2H of the spectrum and errors)
@@ -356,23 +383,11 @@ def run_gpu(args, rank, world, local_rank):
                        + (f", bins shared by groups of {args.shared_bins} walkers" if args.shared_bins else ""), "step": f"one block: {SWEEPS_PER_BLOCK} sweeps x {N_OMEGA} moves x "
                        f"{N_WALKERS} walkers + 2 resyncs + branching", "walkers_per_gpu": N_WALKERS,
                        "l2": "flushed between steps (256 MiB write)", "parallelism": f"{world} independent inversions"},
-            "roofline": {"kernel": "sweep_shared" if args.shared_bins else "sweep_fp32", "bound": "smem",
-                         "achieved": achieved, "peak": smem_gbs, "unit": "GB/s", "frac": achieved / smem_gbs,
-                         "traffic": None if (args.shared_bins or args.index_walk) else kernel_traffic(),
-                         "traffic_note": "DRAM bytes per sweep launch (ncu); the sweep's operands live in shared memory",
+            "roofline": {**rooflines[longest],
+                         **({"other_blocks": rooflines["span" if longest == "tau" else "tau"]} if len(rooflines) > 1 else {}),
                          "peak_source": "measured live in this run (not in MEASURED_PEAKS.json, which has HBM and bf16 only): "
                                         "conflict-free 16-byte shared-memory loads, 2 blocks x 1024 threads per SM",
-                         "algorithmic_bytes_per_move": bytes_per_move, "bytes_per_move_rule": bytes_rule,
-                         "moves_per_launch": moves_per_launch, "launch_ms": sweep_ms / max(sweep_n, 1),
-                         "achieved_rule": "moves_per_launch x algorithmic_bytes_per_move / launch_ms (CUDA events "
-                                          "around every sweep launch on the handle's stream)",
-                         "alu": {"bound": "alu", "achieved": fp32_achieved, "peak": fp32_peak, "unit": "TFLOP/s",
-                                 "frac": fp32_achieved / fp32_peak,
-                                 "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {sm_max_mhz:.0f} MHz",
-                                 "algorithmic_flops_per_move": flops_per_move,
-                                 "flops_per_move_rule": f"{N_TAU} x (9 x (1 - positivity-rejected {pos_frac:.4f}) "
-                                                        f"+ 2 x accepted {acc_frac:.4f})"},
-                         "l2_read_gbs_measured": l2_gbs,
+                         "l2_read_gbs_measured": l2_gbs, "blocks_in_basis": len(part["span"]),
                          "sweep_lanes_per_walker": g.info().get("sweep_lanes"),
                          "sweep_share_of_step": sweep_ms / ms},
             "kernel_ms": {"sweep": sweep_ms, "resync": info1["resync_ms"] - info0["resync_ms"],
