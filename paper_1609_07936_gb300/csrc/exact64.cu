@@ -595,8 +595,8 @@ __device__ int multipliers_at(int N, const double *z, const double *xi, double D
 // the even sum.  A step is then what S grows by if it is even and if it is odd; steps compose, so a
 // scan over the walkers gives S at every walker up to the one whose addition leaves the binade, and
 // that addition is done as such.  One thread's chain of additions (some 60 cycles each) took 0.53 ms
-// at 16384 walkers and 0.07 ms at 2000; this takes a scan for every doubling of the sum past its first
-// 64 terms, 0.14 and 0.02 ms.
+// at 16384 walkers; this takes a scan for every doubling of the sum past its first 64 terms, over a
+// little more than the walkers that double it.
 struct SumStep { unsigned long long even, odd; };
 constexpr unsigned long long kSumTop = 1ull << 53;      // S leaves the binade
 __host__ __device__ __forceinline__ SumStep sum_then(SumStep a, SumStep b) {
@@ -618,43 +618,47 @@ __host__ __device__ __forceinline__ SumStep sum_step(unsigned long long c, int e
     if (rest == half) return {q + (q & 1), q + ((q + 1) & 1)};
     return {q + (rest > half), q + (rest > half)};
 }
-// Where walker l's residue stands in shared memory: threads that read 16, 8 or 4 consecutive ones meet
-// different banks.
+// Where walker l's residue stands in shared memory: threads that read 2^k consecutive ones meet different
+// banks.
 __host__ __device__ __forceinline__ int sum_at(int l) { return l + (l >> 4); }
 
+constexpr int kSumWarps = 8;                           // a scan is short: more warps wait longer for one another
 struct SumShared {
     double s;            // the sum of the first `at` residues
     int at;
-    SumStep warp[32];
+    SumStep warp[kSumWarps];
 };
 // c: N residues at sum_at(l), stored by all threads before a barrier.  Values that are not residues (NaN,
 // negative, huge) and sums below the normal range are added one by one.
-template <int PT>
 __device__ double ordered_sum(const double *c, int N, SumShared &sh) {
+    constexpr int kThreads = 32 * kSumWarps;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int first = tid * PT;
     bool plain = true;
-    for (int l = first; l < min(N, first + PT); ++l) plain = plain && c[sum_at(l)] >= 0.0 && c[sum_at(l)] <= 1e300;
+    for (int l = tid; l < N; l += kSolveThreads) plain = plain && c[sum_at(l)] >= 0.0 && c[sum_at(l)] <= 1e300;
     const bool scan = __syncthreads_and(plain);
     if (tid == 0) {
         double s = 0.0;
-        const int n = scan ? min(N, 64) : N;
+        const int n = scan ? min(N, 32) : N;
         for (int l = 0; l < n; ++l) s += c[sum_at(l)];
         if (!(s >= 1e-290))
             for (int l = n; l < N; ++l) s += c[sum_at(l)];
         sh.s = s;
         sh.at = s >= 1e-290 ? n : N;
     }
-    for (;;) {
-        __syncthreads();
+    auto barrier = [] { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); };
+    while (warp < kSumWarps) {
+        barrier();
         const double s = sh.s;
         const int at = sh.at;
-        if (at >= N) return s;
+        if (at >= N) break;
         const unsigned long long bits = __double_as_longlong(s);
         const int e = (int)(bits >> 52);
         const unsigned long long S = (bits & (kSumTop / 2 - 1)) | kSumTop / 2;
+        // this scan: the walkers up to `end`, each thread some of them
+        const int end = min(N, at + max(kThreads, at + at / 4)), per = (end - at + kThreads - 1) / kThreads;
+        const int first = min(end, at + tid * per), last = min(end, first + per);
         SumStep own = {0, 0};
-        for (int l = max(at, first); l < min(N, first + PT); ++l) own = sum_then(own, sum_step(__double_as_longlong(c[sum_at(l)]), e));
+        for (int l = first; l < last; ++l) own = sum_then(own, sum_step(__double_as_longlong(c[sum_at(l)]), e));
         SumStep incl = own;
         auto up = [&](SumStep v, int o) -> SumStep { return {__shfl_up_sync(kFull, v.even, o), __shfl_up_sync(kFull, v.odd, o)}; };
         for (int o = 1; o < 32; o <<= 1) {
@@ -664,21 +668,19 @@ __device__ double ordered_sum(const double *c, int N, SumShared &sh) {
         if (lane == 31) sh.warp[warp] = incl;
         SumStep before = up(incl, 1);
         if (lane == 0) before = {0, 0};
-        __syncthreads();
-        SumStep w = sh.warp[lane];                      // 32 warps
-        for (int o = 1; o < 32; o <<= 1) {
-            const SumStep t = up(w, o);
-            if (lane >= o) w = sum_then(t, w);
+        barrier();
+        SumStep all = {0, 0}, off = {0, 0};
+        for (int k = 0; k < kSumWarps; ++k) {
+            if (k == warp) off = all;
+            all = sum_then(all, sh.warp[k]);
         }
-        const SumStep all = {__shfl_sync(kFull, w.even, 31), __shfl_sync(kFull, w.odd, 31)};
-        const SumStep off = {__shfl_sync(kFull, w.even, (warp + 31) & 31), __shfl_sync(kFull, w.odd, (warp + 31) & 31)};
-        if (warp > 0) before = sum_then(off, before);
+        before = sum_then(off, before);
         const SumStep after = sum_then(before, own);
         auto at_S = [S](SumStep v) { return S + (S & 1 ? v.odd : v.even); };
         auto value = [e](unsigned long long v) { return __longlong_as_double(((unsigned long long)e << 52) | (v & (kSumTop / 2 - 1))); };
         if (at_S(before) < kSumTop && at_S(after) >= kSumTop) {
             unsigned long long v = at_S(before);
-            for (int l = max(at, first); l < N; ++l) {
+            for (int l = first; l < last; ++l) {
                 const SumStep step = sum_step(__double_as_longlong(c[sum_at(l)]), e);
                 const unsigned long long next = v + (v & 1 ? step.odd : step.even);
                 if (next >= kSumTop) {
@@ -690,9 +692,11 @@ __device__ double ordered_sum(const double *c, int N, SumShared &sh) {
             }
         } else if (tid == 0 && at_S(all) < kSumTop) {
             sh.s = value(at_S(all));
-            sh.at = N;
+            sh.at = end;
         }
     }
+    __syncthreads();
+    return sh.s;
 }
 
 // The whole solve in one block: the search over Delta is sequential, and a trial is cheap because
@@ -813,7 +817,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) branch_solve_kernel(DevProbl
         cmin = c < cmin ? c : cmin;
     }
     // the mean, summed in the oracle's order: where the residues lie close together, z hangs on its last bits
-    const double csum = ordered_sum<PT>(s_chi2, N, s_sum);
+    const double csum = ordered_sum(s_chi2, N, s_sum);
     const double spread = csum / N - cmin;
     const double scale = spread > 0.0 ? 1.0 / spread : 0.0;    // FP64: residues and mean may leave FP32's range, z does not
     const uint2 key = philox_key(P.seed);
