@@ -146,9 +146,8 @@ typedef struct sail_params {
                                same draws and decisions, and with 8 lanes per walker on a uniform
                                tau grid the one-move loop's column values differ from the
                                look-ahead's in the last bits); 0 = choose: look-ahead when the problem has
-                               at least 16 walkers per SM (measured faster there, slower with fewer)
-                               and the last block rejected at least 30% of its proposals for
-                               positivity (measured +12% at 40%, -6% at 22-27%).  Where neither
+                               at least 16 walkers per SM and the last block rejected at least 30% of its proposals for
+                               positivity.  Where neither
                                sweep_loop nor sweep_lanes is given, own-bin blocks in which no
                                decision is expected within FP32's rounding of its threshold run a
                                third loop: the same draws, delta chi2 summed in an orthonormal basis

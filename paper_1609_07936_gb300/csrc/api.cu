@@ -282,8 +282,11 @@ namespace {
 enum { kSweep = 0, kResync = 1, kBranch = 2 };
 
 // Positivity-rejected share of a block's proposals from which the automatic move loop takes the
-// look-ahead loop for the next block (measured on the paper-scale problem: look-ahead +12% at
-// 40% rejections, one move at a time 6% faster at 22-27%).
+// look-ahead loop for the next block.  The line was measured before the one-move loop became one basic
+// block (look-ahead +12% at 40% rejections, one move at a time 6% faster at 22-27%); since then one
+// move at a time is the faster loop above it too (paper-scale problem, 50 sweeps: 21.5 against 23.5 ms
+// at 41%, 21.5 against 27.0 ms at 31%).  It stands because the two loops' columns differ in the last
+// bits on uniform grids: moving it changes results.
 constexpr double kAheadMinPos = 0.30;
 
 // The move loop of the next block: the automatic choice follows the last block's positivity

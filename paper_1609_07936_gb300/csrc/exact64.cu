@@ -1,9 +1,11 @@
 // FP64 kernels whose every operation is rounded on its own (this file is compiled with
 // -fmad=false): the validation sweep, the residual recomputation, the branching solve and
-// imprint, the stochastic average and the state initialisation.  Sums run in the order the
-// method's definition states them (j ascending for a model value, i ascending for chi2,
+// imprint, the stochastic average and the state initialisation.  On an FP64 state sums run in the
+// order the method's definition states them (j ascending for a model value, i ascending for chi2,
 // walkers ascending for an average), so these kernels reproduce a plain sequential FP64
-// evaluation of the same formulas bit for bit, up to the library exp of the Metropolis test.
+// evaluation of the same formulas bit for bit, up to the library exp of the Metropolis test; so does
+// the branching solve for either state.  Averages, smoothing and block statistics of an FP32 state
+// sum in FP64 over lanes, threads or parts of the walkers.
 #include <cfloat>
 #include <cmath>
 #include <cstdint>
@@ -595,8 +597,9 @@ __device__ int multipliers_at(int N, const double *z, const double *xi, double D
 // the even sum.  A step is then what S grows by if it is even and if it is odd; steps compose, so a
 // scan over the walkers gives S at every walker up to the one whose addition leaves the binade, and
 // that addition is done as such.  One thread's chain of additions (some 60 cycles each) took 0.53 ms
-// at 16384 walkers; this takes a scan for every doubling of the sum past its first 64 terms, over a
-// little more than the walkers that double it.
+// at 16384 walkers (block of 512 x 2048, 10 sweeps: 14.80 -> 15.32 ms); this takes a scan for every
+// doubling of the sum past its first 32 terms, over a little more than the walkers that double it
+// (14.90 ms; one solve of 1023 walkers 11 us).
 struct SumStep { unsigned long long even, odd; };
 constexpr unsigned long long kSumTop = 1ull << 53;      // S leaves the binade
 __host__ __device__ __forceinline__ SumStep sum_then(SumStep a, SumStep b) {
@@ -711,7 +714,7 @@ __device__ double ordered_sum(const double *c, int N, SumShared &sh) {
 // for, so FP64 is kept to the walkers' differences from the smallest chi2 and to one warp's
 // scalars.  Against one block per speculative trial in FP64 (23 launches; the same multipliers):
 // 1013 -> 105 us at 4096 walkers, 4050 -> 522 us at 16384, 350 -> 62 us at 1500, 220 -> 28 us at 64
-// (first block of an anneal).
+// (first block of an anneal, the mean summed over threads; its ordered sum, above, comes on top).
 constexpr float kSolveErr = 3e-7f;     // rounding of Theta E + xi and of xi, absolute part
 
 template <int PT>

@@ -27,7 +27,8 @@
 // iteration of four walkers, 290 cycles at two warps on a scheduler, 64% of its issue slots and 67%
 // of the shared-memory data pipe), 16384 walkers 198 -> 45 ms; 512 x 2048 x 16384, 10 sweeps 90 ->
 // 14 ms (spectra in L2); 160 x 1000 x 1500, 100 sweeps 35.5 -> 9.6 ms (203 cycles an iteration,
-// one warp); Hastings 72 -> 15.7 ms; index walk (L = 2, 1500 walkers, 50 sweeps) 47 -> 16 ms.
+// one warp); Hastings 72 -> 15.7 ms; index walk (L = 2, 1500 walkers, 50 sweeps) 47 -> 15 ms.  The
+// warp barrier a move (below) is in the noise of these.
 //
 // Layout.  G lanes per walker (8 or 4: four or eight walkers a warp).  The RR elements belong to
 // eight virtual lanes, RR / 8 each; delta chi2 is the xor-butterfly sum (4, 2, 1) of the virtual
